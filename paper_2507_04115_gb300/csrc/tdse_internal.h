@@ -54,19 +54,22 @@ struct GroupDesc {
                           // scheduler's priority is remaining slices x w
 };
 
-// Device-side tables offsets inside a class block (in doubles).
+// Device-side tables offsets inside a class block (in doubles).  Tables are laid out at the grid size
+// rounded up to even, so that every table (an odd multiple of it among them) starts on the 16 bytes
+// that the double2 and float4 loads need.
+__host__ __device__ inline int64_t tab_n(int N) { return ((int64_t)N + 1) & ~int64_t(1); }
 __host__ __device__ inline int64_t tab_ab(const ClassDesc& c) { return c.tab_off; }
-__host__ __device__ inline int64_t tab_xv(const ClassDesc& c) { return c.tab_off + 2 * (int64_t)c.N; }
-__host__ __device__ inline int64_t tab_mk(const ClassDesc& c) { return c.tab_off + 4 * (int64_t)c.N; }
-__host__ __device__ inline int64_t tab_nw(const ClassDesc& c) { return c.tab_off + 5 * (int64_t)c.N; }
-__host__ __device__ inline int64_t tab_nl(const ClassDesc& c) { return c.tab_off + 7 * (int64_t)c.N; }
-__host__ __device__ inline int64_t tab_nc(const ClassDesc& c) { return c.tab_off + 9 * (int64_t)c.N; }
-__host__ __device__ inline int64_t tab_nf(const ClassDesc& c) { return c.tab_off + 11 * (int64_t)c.N; }
-__host__ __device__ inline int64_t tab_fx(const ClassDesc& c) { return c.tab_off + 14 * (int64_t)c.N; }
-__host__ __device__ inline int64_t tab_vv(const ClassDesc& c) { return c.tab_off + 16 * (int64_t)c.N; }
-__host__ __device__ inline int64_t tab_af(const ClassDesc& c) { return c.tab_off + 17 * (int64_t)c.N; }
-__host__ __device__ inline int64_t tab_xff(const ClassDesc& c) { return c.tab_off + 18 * (int64_t)c.N; }
-inline int64_t tab_doubles(int N) { return 20 * (int64_t)N; }
+__host__ __device__ inline int64_t tab_xv(const ClassDesc& c) { return c.tab_off + 2 * tab_n(c.N); }
+__host__ __device__ inline int64_t tab_mk(const ClassDesc& c) { return c.tab_off + 4 * tab_n(c.N); }
+__host__ __device__ inline int64_t tab_nw(const ClassDesc& c) { return c.tab_off + 5 * tab_n(c.N); }
+__host__ __device__ inline int64_t tab_nl(const ClassDesc& c) { return c.tab_off + 7 * tab_n(c.N); }
+__host__ __device__ inline int64_t tab_nc(const ClassDesc& c) { return c.tab_off + 9 * tab_n(c.N); }
+__host__ __device__ inline int64_t tab_nf(const ClassDesc& c) { return c.tab_off + 11 * tab_n(c.N); }
+__host__ __device__ inline int64_t tab_fx(const ClassDesc& c) { return c.tab_off + 14 * tab_n(c.N); }
+__host__ __device__ inline int64_t tab_vv(const ClassDesc& c) { return c.tab_off + 16 * tab_n(c.N); }
+__host__ __device__ inline int64_t tab_af(const ClassDesc& c) { return c.tab_off + 17 * tab_n(c.N); }
+__host__ __device__ inline int64_t tab_xff(const ClassDesc& c) { return c.tab_off + 18 * tab_n(c.N); }
+inline int64_t tab_doubles(int N) { return 20 * tab_n(N); }
 
 // ---- host-side planning rules shared by the allocating and the static entry points ----
 

@@ -511,6 +511,31 @@ def test_numerov_split_mixed_matches_oracle(env, lanes):
     assert _numerov_case(tdse, oracle, tdse.TDSE_MIXED, lanes=lanes) < MIXED_SERIES
 
 
+@pytest.mark.parametrize("N,lanes", [(401, 1), (401, 8), (1001, 32)])
+def test_numerov_split_fp64_odd_grids(env, N, lanes):
+    """Odd grids: every class table starts on a 16-byte boundary whatever N (the FP64 factors are read
+    as double2), 32-wide and lane-split groups, two classes in one batch."""
+    tdse, oracle = env
+    from paper_2507_04115_gb300 import inputs
+    dx, dt, a, nt = 0.2, 0.05, 1.19, 120
+    sizes = [N, N, 502]
+    rows = [inputs.sin2_pulse(nt, dt, 0.05 + 0.01 * i, 0.057, 1.0, 0.3 * i) for i in range(3)]
+    offs = np.arange(4) * (nt + 1)
+    Et = _device_rows(rows, offs, torch.device("cuda", 0))
+    b = tdse.Batch(sizes, dx, a, nt, dt, absorber=(20.0, 0.125), scheme=tdse.TDSE_NUMEROV_SPLIT, lanes_per_instance=lanes)
+    b.ground_state(**GS_KW)
+    d, acc = torch.zeros_like(Et), torch.zeros_like(Et)
+    b.propagate(Et, d, acc)
+    assert b.check() == -1
+    for i, n in enumerate(sizes):
+        psi0, _, _ = oracle.ground_state(n, dx, a, scheme=oracle.NUMEROV_SPLIT, **GS_KW)
+        _, d_o, a_o = oracle.propagate(psi0, rows[i], dx, dt, a, scheme=oracle.NUMEROV_SPLIT,
+                                       mask_values=oracle.mask(n, dx, 20.0, 0.125))
+        sl = slice(offs[i], offs[i + 1])
+        assert _rel(d[sl].cpu().numpy(), d_o) < RTOL_SERIES and _rel(acc[sl].cpu().numpy(), a_o) < RTOL_SERIES
+    b.close()
+
+
 # ------------------------------------------------------------------------------- adjoint
 
 @pytest.mark.parametrize("lanes", [1, 4])
