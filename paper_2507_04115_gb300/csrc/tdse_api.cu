@@ -130,6 +130,10 @@ struct tdse_batch {
     size_t gtape_bytes = 0;
     bool use_gtape = true;             // tdse_set_adjoint_gamma_tape
     int adj_kc = 0, adj_ctas = 0;
+    // launch shape of the adjoint kernel (its sweeps are in double: the rules of that pipe)
+    std::vector<GroupDesc> adj_groups;
+    GroupDesc* d_adj_groups = nullptr;
+    int adj_warps = 8, adj_rows = 0, adj_grid = 0;
     // checkpoints recorded by tdse_propagate_checkpointed: steps [0, ckpt_next) are covered (-1: none)
     int64_t ckpt_next = -1;
     // energy-distribution buffers (allocated on first use, grown as needed)
@@ -170,6 +174,8 @@ void free_device(tdse_batch* b)
     cudaFree(b->d_slot_group);
     cudaFree(b->d_slot_inst);
     cudaFree(b->d_ed_scratch);
+    cudaFree(b->d_adj_groups);
+    b->d_adj_groups = nullptr;
     b->d_slot_group = b->d_slot_inst = nullptr;
     b->d_ed_scratch = nullptr;
     b->ed_scratch_elems = 0;
@@ -265,6 +271,7 @@ void build_classes(tdse_batch* b, const tdse_instance* inst_host, int64_t n_inst
             C.beta = dt / (4.0 * I.dx * I.dx);
             C.one = 1.0;
             C.nzero = -0.0;
+            C.fix = class_fix(C, dt);
             b->classes.push_back(C);
         } else {
             c = it->second;
@@ -455,38 +462,87 @@ tdse_status build_groups(tdse_batch* b)
     return TDSE_OK;
 }
 
-// (Re)compute the launch configuration, the group descriptors and the scratch, and (re)allocate.
-tdse_status build_plan(tdse_batch* b)
+// Groups of a batch that the fixed-point sweep serves.
+bool on_fix_path(const tdse_batch* b, const ClassDesc& C)
 {
-    const int n_cls = (int)b->classes.size();
-    b->warps = b->warps_override > 0 ? b->warps_override : default_warps(b);
-    b->slice = b->slice_override > 0 ? b->slice_override : 16;
-    b->class_P.assign(n_cls, 1);
-    b->class_K.assign(n_cls, 0);
+    return b->precision == TDSE_FP64 && b->scheme == TDSE_FULL_CN && C.fix.ok;
+}
+
+// Warps, halo, segment length and priority of every group by the FP64 pipe's rules (or, with `fix`, by
+// those of the fixed-point sweep at per_sm CTAs per SM where a class has that form); returns the rows of a
+// sweep's scratch, *widest the warps of a CTA.
+int shape_groups(const tdse_batch* b, std::vector<GroupDesc>& groups, bool fix, int per_sm, int* widest)
+{
+    const int most = b->warps_override > 0 ? b->warps_override : default_warps(b);
+    const int most_fix = b->warps_override > 0 ? most : kMaxSegments / per_sm;
     int rows = 1;
-    for (auto& G : b->groups) {
+    *widest = 1;
+    for (auto& G : groups) {
         const ClassDesc& C = b->classes[G.cls];
         const int L = kLanes / G.I;
         int K = class_halo(b, C);
-        const int P = group_warps(C.N, K, L, b->warps);
+        const bool fx = fix && on_fix_path(b, C);
+        const int cap = fix && b->warps_override <= 0 ? std::min(most, most_fix) : most;
+        const int P = fx ? fix_warps(C.N, K, L, most_fix, per_sm) : group_warps(C.N, K, L, cap);
         if (P == 1 && L == 1) K = 0;   // one exact segment
         G.P = P;
         G.K = K;
         G.m = group_segment_length(G.N, P, L);
-        G.w = std::max(1, (int)std::lround(group_step_cost(C.N, K, L, b->warps) / 64.0));
-        b->class_P[G.cls] = std::max(b->class_P[G.cls], P);
-        b->class_K[G.cls] = std::max(b->class_K[G.cls], K);
+        G.w = std::max(1, (int)std::lround((fx ? fix_step_cost(C.N, K, L, P, P * per_sm) : group_step_cost(C.N, K, L, cap)) / 64.0));
+        *widest = std::max(*widest, fx ? P : cap);
         // a sweep covers its segment and a halo on each side (m + 2K rows; the 32-wide propagation
         // clips it at the walls); a single exact segment covers the N points
-        rows = std::max(rows, P * (kLanes / G.I) == 1 ? G.N : G.m + 2 * K);
+        rows = std::max(rows, P * L == 1 ? G.N : G.m + 2 * K);
     }
-    b->rows = rows;
+    if (b->warps_override > 0) *widest = most;
+    return rows;
+}
+
+// (Re)compute the launch configuration, the group descriptors and the scratch, and (re)allocate.
+tdse_status build_plan(tdse_batch* b)
+{
+    const int n_cls = (int)b->classes.size();
+    b->slice = b->slice_override > 0 ? b->slice_override : 16;
+    bool fix = false;
+    for (const ClassDesc& C : b->classes) fix = fix || on_fix_path(b, C);
+    int want = 1;
+    if (b->ctas_per_sm_override > 0)
+        want = b->ctas_per_sm_override;
+    else if (fix && b->warps_override <= 0) {
+        std::vector<FixGroup> g;
+        for (const GroupDesc& G : b->groups)
+            g.push_back({G.N, class_halo(b, b->classes[G.cls]), kLanes / G.I, (double)std::max<int64_t>(G.nt_max, 1)});
+        want = fix_ctas_per_sm(g, b->sm_count);
+    }
+    const int shape_per_sm = want >= 4 ? 4 : (want >= 2 ? 2 : 1);
+    b->rows = shape_groups(b, b->groups, fix, shape_per_sm, &b->warps);
+    b->class_P.assign(n_cls, 1);
+    b->class_K.assign(n_cls, 0);
+    for (const GroupDesc& G : b->groups) {
+        b->class_P[G.cls] = std::max(b->class_P[G.cls], G.P);
+        b->class_K[G.cls] = std::max(b->class_K[G.cls], G.K);
+    }
     const int per_sm_max = propagate_max_ctas_per_sm(b->mixed(), b->warps);
-    const int per_sm = b->ctas_per_sm_override > 0 ? std::min(b->ctas_per_sm_override, per_sm_max) : 1;
+    const int per_sm = std::min(want, per_sm_max);
     b->ring = propagate_ring_slots(b->warps, per_sm);
-    b->ctas = (int)std::min<int64_t>((int64_t)b->groups.size(), (int64_t)b->sm_count * per_sm);
-    if (b->max_ctas_override > 0) b->ctas = std::min(b->ctas, b->max_ctas_override);
-    const int64_t sc = (int64_t)b->ctas * b->warps * rows * 2 * kLanes;
+    auto grid = [&](int k) {
+        const int64_t n = std::min<int64_t>((int64_t)b->groups.size(), (int64_t)b->sm_count * k);
+        return (int)(b->max_ctas_override > 0 ? std::min<int64_t>(n, b->max_ctas_override) : n);
+    };
+    b->ctas = grid(per_sm);
+    int64_t sc = (int64_t)b->ctas * b->warps * b->rows * 2 * kLanes;
+    if (b->precision == TDSE_FP64 && b->scheme == TDSE_FULL_CN) {
+        // the adjoint kernel's shape; it shares the scratch
+        b->adj_groups = b->groups;
+        b->adj_rows = shape_groups(b, b->adj_groups, false, 1, &b->adj_warps);
+        b->adj_grid = grid(b->ctas_per_sm_override > 0 ? std::min(b->ctas_per_sm_override, propagate_max_ctas_per_sm(0, b->adj_warps)) : 1);
+        sc = std::max(sc, (int64_t)b->adj_grid * b->adj_warps * b->adj_rows * 2 * kLanes);
+        cudaFree(b->d_adj_groups);
+        b->d_adj_groups = nullptr;
+        TDSE_CUDA(dev_alloc(&b->d_adj_groups, b->adj_groups.size()), "cudaMalloc(groups)");
+        TDSE_CUDA(cudaMemcpy(b->d_adj_groups, b->adj_groups.data(), sizeof(GroupDesc) * b->adj_groups.size(), cudaMemcpyHostToDevice),
+                  "cudaMemcpy(groups)");
+    }
     cudaFree(b->d_scratch);
     b->d_scratch = nullptr;
     TDSE_CUDA(cudaMalloc(&b->d_scratch, (size_t)std::max<int64_t>(sc, 1) * b->cx_bytes()), "cudaMalloc(scratch)");
@@ -510,7 +566,7 @@ tdse_status ensure_adjoint_buffers(tdse_batch* b, int ckpt_every, cudaStream_t s
     int n_max = 1;
     for (auto& G : b->groups) n_max = std::max(n_max, G.N);
     *n_max_out = n_max;
-    if (!b->d_lam || b->adj_kc != ckpt_every || b->adj_ctas != b->ctas) {
+    if (!b->d_lam || b->adj_kc != ckpt_every || b->adj_ctas != b->adj_grid) {
         b->ckpt_next = -1;
         TDSE_CUDA(cudaStreamSynchronize(st), "tdse_adjoint: synchronize");
         cudaFree(b->d_lam);
@@ -532,13 +588,13 @@ tdse_status ensure_adjoint_buffers(tdse_batch* b, int ckpt_every, cudaStream_t s
         TDSE_CUDA(cudaMalloc(&b->d_lam, (size_t)std::max<int64_t>(b->psi_elems, 1) * cx), "cudaMalloc(adjoint lambda)");
         TDSE_CUDA(cudaMalloc(&b->d_ckpt, (size_t)std::max<int64_t>(total, 1) * cx), "cudaMalloc(adjoint checkpoints)");
         TDSE_CUDA(dev_alloc(&b->d_ckpt_off, off.size()), "cudaMalloc(adjoint offsets)");
-        TDSE_CUDA(cudaMalloc(&b->d_work, (size_t)b->ctas * n_max * kLanes * cx), "cudaMalloc(adjoint work)");
-        TDSE_CUDA(cudaMalloc(&b->d_tape, (size_t)b->ctas * ckpt_every * (size_t)n_max * kLanes * cx),
+        TDSE_CUDA(cudaMalloc(&b->d_work, (size_t)b->adj_grid * n_max * kLanes * cx), "cudaMalloc(adjoint work)");
+        TDSE_CUDA(cudaMalloc(&b->d_tape, (size_t)b->adj_grid * ckpt_every * (size_t)n_max * kLanes * cx),
                   "cudaMalloc(adjoint tape)");
         TDSE_CUDA(cudaMemcpy(b->d_ckpt_off, off.data(), sizeof(int64_t) * off.size(), cudaMemcpyHostToDevice),
                   "cudaMemcpy(adjoint offsets)");
         b->adj_kc = ckpt_every;
-        b->adj_ctas = b->ctas;
+        b->adj_ctas = b->adj_grid;
     }
     return TDSE_OK;
 }
@@ -549,7 +605,7 @@ tdse_status ensure_adjoint_buffers(tdse_batch* b, int ckpt_every, cudaStream_t s
 // without it): allocated when it takes at most half of the device's free memory, else left out.
 void ensure_gamma_tape(tdse_batch* b, int kc)
 {
-    const size_t need = (size_t)b->ctas * kc * (size_t)b->warps * b->rows * kLanes * sizeof(double2);
+    const size_t need = (size_t)b->adj_grid * kc * (size_t)b->adj_warps * b->adj_rows * kLanes * sizeof(double2);
     if (b->d_gtape && b->gtape_bytes == need) return;
     cudaFree(b->d_gtape);
     b->d_gtape = nullptr;
@@ -626,7 +682,7 @@ tdse_status tdse_batch_create(const tdse_instance* inst_host, int64_t n_inst, do
     int max_N = 0;
     for (auto& C : b->classes) {
         C.tab_off = tab_total;
-        tab_total += tab_doubles(C.N);
+        tab_total += tab_doubles(C);
         max_N = std::max(max_N, C.N);
         C.jm_lo = 0;
         C.jm_hi = C.N - 1;
@@ -986,9 +1042,9 @@ tdse_status tdse_adjoint(tdse_batch* b, const double* E_dev, const double* gd_de
     if (s != TDSE_OK) return s;
     b->ckpt_next = -1;   // the adjoint's own forward pass rewrites the checkpoints
     if (b->use_gtape) ensure_gamma_tape(b, ckpt_every);
-    TDSE_CUDA(launch_adjoint_full_cn(b->d_groups, (int64_t)b->groups.size(), b->warps, b->ctas, b->d_cls, b->d_tab,
+    TDSE_CUDA(launch_adjoint_full_cn(b->d_adj_groups, (int64_t)b->groups.size(), b->adj_warps, b->adj_grid, b->d_cls, b->d_tab,
                                      b->d_slot_row, b->d_slot_nt, b->d_psi, b->d_lam, b->d_ckpt, b->d_ckpt_off,
-                                     b->d_work, b->d_tape, b->d_scratch, b->rows, n_max, ckpt_every, E_dev, gd_dev,
+                                     b->d_work, b->d_tape, b->d_scratch, b->adj_rows, n_max, ckpt_every, E_dev, gd_dev,
                                      ga_dev, gE_dev, b->mask_on, b->d_busy, b->d_progress, st, 0,
                                      b->use_gtape ? b->d_gtape : nullptr),
               "adjoint launch");
@@ -1049,9 +1105,9 @@ tdse_status tdse_adjoint_checkpointed(tdse_batch* b, const double* E_dev, const 
         return fail(TDSE_ERR_STATE, "tdse_adjoint_checkpointed: no complete checkpointed forward propagation "
                                     "(tdse_propagate_checkpointed from step 0 through every instance's last step)");
     if (b->use_gtape) ensure_gamma_tape(b, b->adj_kc);
-    TDSE_CUDA(launch_adjoint_full_cn(b->d_groups, (int64_t)b->groups.size(), b->warps, b->ctas, b->d_cls, b->d_tab,
+    TDSE_CUDA(launch_adjoint_full_cn(b->d_adj_groups, (int64_t)b->groups.size(), b->adj_warps, b->adj_grid, b->d_cls, b->d_tab,
                                      b->d_slot_row, b->d_slot_nt, b->d_psi, b->d_lam, b->d_ckpt, b->d_ckpt_off,
-                                     b->d_work, b->d_tape, b->d_scratch, b->rows, n_max, b->adj_kc, E_dev, gd_dev,
+                                     b->d_work, b->d_tape, b->d_scratch, b->adj_rows, n_max, b->adj_kc, E_dev, gd_dev,
                                      ga_dev, gE_dev, b->mask_on, b->d_busy, b->d_progress, st, 1,
                                      b->use_gtape ? b->d_gtape : nullptr),
               "adjoint launch");

@@ -23,7 +23,7 @@
 //     (8192 instances = 256 groups on 152 SMs) and when groups have different lengths.
 // HBM layouts: psi [group][j][lane] (16 B per point, a warp reads 512 contiguous bytes), scratch per
 // CTA [warp][row][gamma | D][lane].
-#include "tdse_sched.cuh"
+#include "tdse_cn_fix.cuh"
 
 namespace tdse {
 
@@ -311,7 +311,14 @@ k_propagate_full_cn(const GroupDesc* __restrict__ groups, int64_t n_groups, cons
         const int64_t n0 = step_begin + (int64_t)kslice * slice;
         const int64_t n1 = min(n_end, n0 + slice);
 
-        if (G.I != kLanes) {
+        bool done = false;
+        if constexpr (!kMixed)
+            if (fix_shape(G, C))
+                done = fix_slice<kCkpt>(G, C, tab, ps, nt, row, slot, n0, n1, kslice == 0 && step_begin == 0, E, d_out, a_out,
+                                        sample_base, reinterpret_cast<int4*>(scratch_raw) + (int64_t)blockIdx.x * P * rows * (2 * kLanes),
+                                        red, status, kCkpt ? ckpt + ckpt_off[g] : nullptr, kc, jm_lo, jm_hi);
+        if (done) {
+        } else if (G.I != kLanes) {
             split_slice<kMixed, kCkpt>(G, F, ps, tab_ab2, tab_xv2, tab_m, inv_beta, two_over_beta, dx, jm_lo, jm_hi,
                                        nt, row, slot, n0, n1, kslice == 0 && step_begin == 0, E, d_out, a_out,
                                        sample_base, sc, red, status, kCkpt ? ckpt + ckpt_off[g] : nullptr, kc,

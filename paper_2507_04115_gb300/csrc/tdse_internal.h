@@ -10,6 +10,7 @@
 #include <cuda_runtime.h>
 
 #include "tdse.h"
+#include "tdse_fix.cuh"
 
 namespace tdse {
 
@@ -28,6 +29,7 @@ constexpr int kMaxSegments = 16;    // warps per CTA at most (512 threads)
 //   af[j]  = ab[j] rounded to float2                                      (float halo rows)
 //   xff[j] = (x_j, dV_j) as float pairs (hi, lo), hi = x rounded to float, lo = x - hi rounded
 //            to float: a float4 (x_hi, x_lo, dV_hi, dV_lo)
+//   fxp[j] = FixPoint, fob[j] = FixObs: the fixed-point sweep's tables (classes with fix.ok)
 struct ClassDesc {
     int64_t tab_off;      // offset (in doubles) of the class block in the table buffer
     int32_t N;
@@ -36,6 +38,7 @@ struct ClassDesc {
     double beta;          // dt / (4 dx^2): magnitude of the off-diagonal of 1 + i dt/2 H
     double rho;           // NUMEROV_SPLIT: max_j max(|L_j|, |C_j|), the decay rate of its sweeps
     double one, nzero;    // 1.0 and -0.0 as data, for adds and multiplies issued as FMAs (Fma64)
+    FixClass fix;         // fixed-point form of the FULL_CN sweep (tdse_fix.cuh)
 };
 
 // A group = I instances of one class.  With I = 32 every lane of a warp carries its own instance;
@@ -69,9 +72,19 @@ __host__ __device__ inline int64_t tab_fx(const ClassDesc& c) { return c.tab_off
 __host__ __device__ inline int64_t tab_vv(const ClassDesc& c) { return c.tab_off + 16 * tab_n(c.N); }
 __host__ __device__ inline int64_t tab_af(const ClassDesc& c) { return c.tab_off + 17 * tab_n(c.N); }
 __host__ __device__ inline int64_t tab_xff(const ClassDesc& c) { return c.tab_off + 18 * tab_n(c.N); }
-inline int64_t tab_doubles(int N) { return 20 * tab_n(N); }
+__host__ __device__ inline int64_t tab_fxp(const ClassDesc& c) { return c.tab_off + 20 * tab_n(c.N); }
+__host__ __device__ inline int64_t tab_fob(const ClassDesc& c) { return c.tab_off + 22 * tab_n(c.N); }
+inline int64_t tab_doubles(const ClassDesc& c) { return (c.fix.ok ? 24 : 20) * tab_n(c.N); }
 
 // ---- host-side planning rules shared by the allocating and the static entry points ----
+
+// Fixed-point form of a class: |V| <= |Z| / a and |dV/dx| <= 2 |Z| / (3 sqrt(3) a^2) over the grid.
+inline FixClass class_fix(const ClassDesc& c, double dt)
+{
+    const double d2 = 2.0 * c.dx * c.dx;
+    return fix_class(c.N, c.dx, dt, 2.0 + d2 * std::fabs(c.Z) / c.a, d2 * 0.5 * (c.N - 1) * c.dx,
+                     0.385 * std::fabs(c.Z) / (c.a * c.a));
+}
 
 // Halo length K such that beta^K < tol (1e-18 by default): the truncated sweeps then agree with the
 // exact Thomas solve below double rounding (|gamma| <= |beta| per point, see tdse_full_cn.cu); 0 when
@@ -116,6 +129,60 @@ inline double group_step_cost(int N, int K, int L, int warps)
     const int P = group_warps(N, K, L, warps);
     const int m = group_segment_length(N, P, L);
     return std::ceil(P / 4.0) * (27.0 * m + 36.0 * (P * L > 1 ? K : 0));
+}
+
+// Step of a group on the fixed-point sweep (tdse_cn_fix.cuh), in the unit of group_step_cost: every warp
+// runs m + 1.3 K rows (the lead-in's K back substitutions and K whole rows), and a row takes 6 + W
+// units, W the warps that share the SM (at least 4, one per sub-partition): its latency, hidden by the
+// other warps as far as they are, and everyone's instructions.  Measured, volume batch (K = 28, 160
+// steps): 120 ms at 8 warps, 104 at 12, 100 at 16, 113 with two CTAs of 8; one atom (K = 36, L = 32, 512
+// steps): 23.7 ms at 2 warps, 18.8 at 4, 20.9 at 8.
+inline double fix_step_cost(int N, int K, int L, int P, int W)
+{
+    const int m = group_segment_length(N, P, L);
+    return 0.17 * (6.0 + std::max(W, 4)) * (m + 1.3 * (P * L > 1 ? K : 0));
+}
+// Warps carrying segments there when `per_sm` CTAs share an SM: the cheapest of those that group_warps
+// allows, segments of at least 4 points (a pass reads its own rows three ahead).
+inline int fix_warps(int N, int K, int L, int warps, int per_sm)
+{
+    int best = 1;
+    for (int P = 2; P <= group_warps(N, K, L, warps); ++P)
+        if (group_segment_length(N, P, L) >= 4 &&
+            fix_step_cost(N, K, L, P, P * per_sm) < fix_step_cost(N, K, L, best, best * per_sm)) best = P;
+    return best;
+}
+
+// CTAs per SM (1, 2 or 4, of at most 16 / per_sm warps: 128 registers a thread) for a batch on the
+// fixed-point sweep: fewer, longer segments per instance carry less halo, and more CTAs hide the
+// latency, where there are groups enough to fill them.  The estimate is the makespan: the work over the
+// SMs, and the longest group at the pace it has beside its neighbours.  Measured: 625 groups of N = 1024
+// take 43.3 ms at 1 x 9 warps, 29.1 at 2 x 8, 26.4 at 4 x 4; 304 groups of 4096 47.9 at 1 x 16 and 45.5 at
+// 2 x 8; 256 of them 100 at 1 x 16 and 113 at 2 x 8.
+struct FixGroup {
+    int N, K, L;
+    double nt;
+};
+inline int fix_ctas_per_sm(const std::vector<FixGroup>& groups, int sm_count)
+{
+    double best_t = 0.0;
+    int best = 1;
+    for (int c = 1; c <= 4; c *= 2) {
+        double work = 0.0, longest = 0.0;
+        const int share = (int)std::min<int64_t>(c, ((int64_t)groups.size() + sm_count - 1) / sm_count);
+        for (const FixGroup& g : groups) {
+            const int P = fix_warps(g.N, g.K, g.L, kMaxSegments / c, c);
+            const double t = g.nt * fix_step_cost(g.N, g.K, g.L, P, P * share);
+            work += t / share;
+            longest = std::max(longest, t);
+        }
+        const double t = std::max(work / std::max(1, sm_count), longest);
+        if (c == 1 || t < 0.97 * best_t) {
+            best_t = t;
+            best = c;
+        }
+    }
+    return best;
 }
 
 // Group widths by the whole job's makespan.  A group of instances with Nt_max steps keeps one SM

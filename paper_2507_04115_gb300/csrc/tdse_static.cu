@@ -116,6 +116,7 @@ extern "C" tdse_status tdse_propagate_static(const tdse_instance* inst_host, int
     C.beta = dt / (4.0 * I.dx * I.dx);
     C.one = 1.0;
     C.nzero = -0.0;
+    C.fix = class_fix(C, dt);
     C.tab_off = 0;
     const int mask_on = absorber && absorber->width > 0.0;
     C.jm_lo = 0;
@@ -155,7 +156,7 @@ extern "C" tdse_status tdse_propagate_static(const tdse_instance* inst_host, int
     const size_t o_busy = take(sizeof(int) * (size_t)n_groups);
     const size_t o_prog = take(sizeof(int) * (size_t)n_groups);
     const size_t o_status = take(sizeof(int) * (size_t)n_groups * kLanes);
-    const size_t o_tab = take(sizeof(double) * (size_t)tab_doubles(C.N));
+    const size_t o_tab = take(sizeof(double) * (size_t)tab_doubles(C));
     const size_t o_scratch = off;
     const size_t per_cta = sizeof(double2) * (size_t)warps * rows * 2 * kLanes;
     if (o_scratch >= kStaticBytes || (kStaticBytes - o_scratch) / per_cta < 1) {

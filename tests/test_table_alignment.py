@@ -17,13 +17,16 @@ int main() {
         ClassDesc c{};
         c.N = N;
         c.tab_off = base;
+        c.fix.ok = 1;
         const int64_t at[] = {tab_ab(c), tab_xv(c), tab_mk(c), tab_nw(c), tab_nl(c), tab_nc(c),
-                              tab_nf(c), tab_fx(c), tab_vv(c), tab_af(c), tab_xff(c), base + tab_doubles(N)};
-        const int64_t len[] = {2, 2, 1, 2, 2, 2, 3, 2, 1, 1, 2};   // doubles per point
-        for (int k = 0; k < 11; ++k)
+                              tab_nf(c), tab_fx(c), tab_vv(c), tab_af(c), tab_xff(c), tab_fxp(c), tab_fob(c), base + tab_doubles(c)};
+        const int64_t len[] = {2, 2, 1, 2, 2, 2, 3, 2, 1, 1, 2, 2, 2};   // doubles per point
+        for (int k = 0; k < 13; ++k)
             if (at[k] % 2 != 0 || at[k] + len[k] * N > at[k + 1]) return 1 + k;
-        base += tab_doubles(N);
+        base += tab_doubles(c);
         if (base % 2) return 20;
+        c.fix.ok = 0;   // classes without the fixed-point form end before its tables
+        if (tab_doubles(c) > tab_fxp(c) - c.tab_off) return 21;
     }
     return 0;
 }
