@@ -1267,6 +1267,20 @@ tdse_status tdse_spectrum(const double* a_dev, const int64_t* offsets_host, int6
         if (offsets_host[r + 1] < offsets_host[r] || offsets_host[r] < 0)
             return fail(TDSE_ERR_ARG, "tdse_spectrum: offsets must be non-decreasing and >= 0");
     cudaStream_t st = (cudaStream_t)stream;
+    // a band far below the sampling rate, every bin below half of the shortest row: by block moments
+    int64_t shortest = offsets_host[1] - offsets_host[0], longest = shortest;
+    for (int64_t r = 1; r < n_rows; ++r) {
+        const int64_t L = offsets_host[r + 1] - offsets_host[r];
+        shortest = std::min(shortest, L);
+        longest = std::max(longest, L);
+    }
+    int B = 0, P = 0;
+    if (shortest > 0 && longest < (int64_t(1) << 30) && 2 * (k_end - 1) < shortest &&
+        dft_plan(shortest, 2.0 * 3.14159265358979323846 * (double)(k_end - 1) / (double)shortest, k_end - k_begin, &B, &P)) {
+        TDSE_CUDA(launch_band_dft(a_dev, offsets_host, n_rows, dt, nullptr, k_begin, k_end - k_begin, B, P, nullptr, S_dev, st),
+                  "tdse_spectrum");
+        return TDSE_OK;
+    }
     int64_t* d_off = nullptr;
     TDSE_CUDA(cudaMallocAsync(reinterpret_cast<void**>(&d_off), sizeof(int64_t) * (n_rows + 1), st), "cudaMallocAsync(offsets)");
     cudaError_t e = cudaMemcpyAsync(d_off, offsets_host, sizeof(int64_t) * (n_rows + 1), cudaMemcpyHostToDevice, st);

@@ -180,6 +180,15 @@ extern "C" tdse_status tdse_dipole_spectrum(const double* a_dev, const int64_t* 
         if (!std::isfinite(omega_host[w]) || std::fabs(omega_host[w]) > 1e6)
             return arg_error("tdse_dipole_spectrum: frequency " + std::to_string(w) + " not finite or beyond 1e6");
     cudaStream_t st = (cudaStream_t)stream;
+    double turn = 0.0;
+    for (int w = 0; w < n_omega; ++w) turn = std::max(turn, std::fabs(omega_host[w]) * dt);
+    int64_t longest = 0;
+    for (int64_t r = 0; r < n_rows; ++r) longest = std::max(longest, offsets_host[r + 1] - offsets_host[r]);
+    int B = 0, P = 0;
+    if (dft_plan(longest, turn, n_omega, &B, &P)) {   // frequencies far below the sampling rate: by block moments
+        const cudaError_t eb = launch_band_dft(a_dev, offsets_host, n_rows, dt, omega_host, 0, n_omega, B, P, weight_dev, out_dev, st);
+        return eb == cudaSuccess ? TDSE_OK : cuda_error(eb, "tdse_dipole_spectrum");
+    }
     int64_t* d_off = nullptr;
     double* d_om = nullptr;
     cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&d_off), sizeof(int64_t) * (n_rows + 1), st);

@@ -369,6 +369,14 @@ cudaError_t launch_get_psi(int mixed, const void* d_psi, int64_t psi_off, int N,
                            cudaStream_t st);
 cudaError_t launch_set_psi(int mixed, void* d_psi, int64_t psi_off, int N, int lane, int I, const double* in, cudaStream_t st);
 
+// Fourier sums by Chebyshev block moments (tdse_dft.cu).  dft_plan: block length and number of moments for
+// rows of `samples` samples at n_w frequencies that turn by at most `turn` rad a sample; false where the
+// direct sum is the better one.  launch_band_dft: omega_host given: weighted complex sums as
+// tdse_dipole_spectrum; NULL: the power spectrum at bins k_begin .. k_begin + n_w - 1 of every row.
+bool dft_plan(int64_t samples, double turn, int64_t n_w, int* B, int* P);
+cudaError_t launch_band_dft(const double* a, const int64_t* offs_host, int64_t n_rows, double dt, const double* omega_host,
+                            int64_t k_begin, int64_t n_w, int B, int P, const double* weight, double* out, cudaStream_t st);
+
 cudaError_t launch_spectrum(const double* a, const int64_t* d_offsets, int64_t n_rows, double dt, int64_t k_begin,
                             int64_t k_end, double* S, cudaStream_t st);
 
