@@ -1246,12 +1246,14 @@ tdse_status tdse_resample_field(const double* coarse_dev, int64_t n_rows, int32_
     DeviceGuard guard(device);
     if (!guard.ok) return fail(TDSE_ERR_CUDA, "cudaSetDevice failed");
     cudaStream_t st = (cudaStream_t)stream;
-    void* d_coef = nullptr;
-    cudaError_t e = cudaMalloc(&d_coef, sizeof(double2) * (size_t)n_rows * (M / 2 + 1));
-    if (e == cudaSuccess) e = launch_resample_field(coarse_dev, n_rows, M, dt_coarse, dt_fine, n_fine, out_stride, out_dev,
-                                                    d_coef, st);
+    void* d_work = nullptr;
+    cudaError_t e = cudaMallocAsync(&d_work, resample_field_bytes(resample_field_rows(n_rows, M), M, n_fine), st);
+    if (e == cudaSuccess) {
+        e = launch_resample_field(coarse_dev, n_rows, M, dt_coarse, dt_fine, n_fine, out_stride, out_dev, d_work, st);
+        const cudaError_t f = cudaFreeAsync(d_work, st);
+        if (e == cudaSuccess) e = f;
+    }
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    cudaFree(d_coef);
     if (e != cudaSuccess) return cuda_fail(e, "tdse_resample_field");
     return TDSE_OK;
 }

@@ -35,3 +35,17 @@ def test_resample_matches_oracle(env, M, dt_c, dt_f, n_fine):
         ref = oracle.resample_field(coarse[r], dt_c, dt_f, n_fine)
         assert np.max(np.abs(got[r, :n_fine] - ref)) < 1e-12 * max(1.0, np.max(np.abs(coarse[r])))
         assert np.all(got[r, n_fine:] == 0.0)   # the stride padding is left alone
+
+
+@pytest.mark.parametrize("M,n_rows,n_fine", [(8192, 3, 5000), (3, 9, 200), (63, 17, 1000), (65, 8, 257), (16, 1, 100)])
+def test_resample_edges(env, M, n_rows, n_fine):
+    """The largest and the smallest rows (shared memory, the smallest oversampled grid), row counts around
+    the rows of a thread, output counts around a block, outputs past the window."""
+    tdse, oracle = env
+    rng = np.random.default_rng(M + n_rows)
+    coarse = rng.standard_normal((n_rows, M))
+    dt_c, dt_f = 0.5, 0.5 * 1.3 * M / n_fine
+    got = tdse.resample_field(torch.from_numpy(coarse).to("cuda"), dt_c, dt_f, n_fine).cpu().numpy()
+    for r in range(n_rows):
+        ref = oracle.resample_field(coarse[r], dt_c, dt_f, n_fine)
+        assert np.max(np.abs(got[r] - ref)) < 2e-11 * np.max(np.abs(coarse[r]))
