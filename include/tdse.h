@@ -195,7 +195,8 @@ tdse_status tdse_check(tdse_batch* batch, int64_t* first_bad_host, void* stream)
  *   P_dev         out: n_inst x n_energies doubles, row i = instance i in creation order
  * Works on FP64 and MIXED batches (the solves always run in FP64).  Synchronous: allocates the
  * pivot tables (2 x 16 B x N x n_energies per class) for the call, keeps a solve scratch of
- * 8 x SMs x 32 x N_max x 16 B on the batch, and synchronises the stream before returning. */
+ * 16 x SMs x 32 x N_max x 16 B on the batch (8 x where that is above 8 GB), and synchronises the stream
+ * before returning. */
 tdse_status tdse_energy_distribution(tdse_batch* batch, const double* E_grid_host, int32_t n_energies,
                                      double epsilon, double* P_dev, void* stream);
 

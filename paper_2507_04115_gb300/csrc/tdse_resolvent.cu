@@ -16,8 +16,8 @@
 //   k_ed_solve   one warp per (instance, block of 32 energies), one lane per energy:
 //                d'_j = (r_j - a_j d'_{j-1}) / w_j forward (r = M psi), y_j = d'_j - c'_j y_{j+1}
 //                backward, summing |y_j|^2; d' rows go to a per-warp scratch [j][lane].
-// Work per point of a (instance, energy) solve: 13 FP64 operations (the pivot work is amortised
-// over the class's instances).
+// Work per point of a (instance, energy) solve: 10 FP64 instructions (12 on the Numerov pencil), the pivot
+// work amortised over the class's instances.
 #include "tdse_sched.cuh"
 
 namespace tdse {
@@ -79,21 +79,30 @@ __global__ void k_ed_pivots(const ClassDesc* __restrict__ cls, int n_cls, const 
         const double2 ac = cmul(r.a, cprev);
         const double2 w = make_double2(r.b.x - ac.x, r.b.y - ac.y);
         const double2 iw = cinv(w);
-        cprev = cmul(r.c, iw);
-        W[(int64_t)j * nE_pad + k] = iw;
+        if (scheme == 0) {   // a / w_j, which is c'_j but for the last row (see k_ed_solve)
+            const double a = 0.5 * inv_dx2;
+            cprev = make_double2(a * iw.x, a * iw.y);
+        } else {
+            cprev = cmul(r.c, iw);
+            W[(int64_t)j * nE_pad + k] = iw;
+        }
         Cp[(int64_t)j * nE_pad + k] = cprev;
     }
 }
 
-template <class Cx>
+// FULL_CN (kScheme 0): the off-diagonals are one real number a, so with D = a d' and Y = a y the sweeps are
+//     D_j = c'_j (r_j - D_{j-1}),  Y_j = D_j - c'_j Y_{j+1},  c'_j = a / w_j,
+// 10 FP64 instructions a point and one table, and |y|^2 = |Y|^2 / a^2.
+template <class Cx, int kScheme>
 __global__ void k_ed_solve(const GroupDesc* __restrict__ groups, const ClassDesc* __restrict__ cls,
                            const double* __restrict__ tab, const int64_t* __restrict__ slot_group,
                            const int64_t* __restrict__ slot_inst, int64_t n_slots, const Cx* __restrict__ psi_all,
-                           const double* __restrict__ E_grid, int nE, int nE_pad, double eps, int scheme,
+                           const double* __restrict__ E_grid, int nE, int nE_pad, double eps,
                            const double2* __restrict__ pivW, const double2* __restrict__ pivC,
                            const int64_t* __restrict__ piv_off, double2* __restrict__ scratch, int n_max,
                            double* __restrict__ P_out)
 {
+    constexpr int scheme = kScheme;
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t n_warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -114,7 +123,7 @@ __global__ void k_ed_solve(const GroupDesc* __restrict__ groups, const ClassDesc
         const double zr = k < nE ? E_grid[k] : 0.0, zi = -eps;
         const double inv_dx2 = 1.0 / (C.dx * C.dx);
         const double* V = tab + tab_vv(C);
-        const double2* W = pivW + piv_off[G.cls] + k;
+        const double2* W = (scheme == 0 ? pivC : pivW) + piv_off[G.cls] + k;   // the forward sweep's factors
         const double2* Cp = pivC + piv_off[G.cls] + k;
         // forward: d'_j = (r_j - a_j d'_{j-1}) / w_j
         double dr = 0.0, di = 0.0;
@@ -131,16 +140,17 @@ __global__ void k_ed_solve(const GroupDesc* __restrict__ groups, const ClassDesc
                 rr = k12 * fma(10.0, (double)pc.x, F.add((double)pm.x, (double)pn.x));
                 ri = k12 * fma(10.0, (double)pc.y, F.add((double)pm.y, (double)pn.y));
             }
-            double2 a;
-            if (scheme == 0) {
-                a = make_double2(j > 0 ? 0.5 * inv_dx2 : 0.0, 0.0);
-            } else {
-                a = j > 0 ? make_double2(fma(zr, 1.0 / 12.0, 0.5 * inv_dx2 - V[j - 1] * (1.0 / 12.0)), zi * (1.0 / 12.0))
-                          : make_double2(0.0, 0.0);
-            }
             // u = r - a d'
-            const double ur = fma(-a.x, dr, fma(a.y, di, rr));
-            const double ui = fma(-a.x, di, fma(-a.y, dr, ri));
+            double ur, ui;
+            if (scheme == 0) {
+                ur = F.sub(rr, dr);
+                ui = F.sub(ri, di);
+            } else {
+                const double2 a = j > 0 ? make_double2(fma(zr, 1.0 / 12.0, 0.5 * inv_dx2 - V[j - 1] * (1.0 / 12.0)), zi * (1.0 / 12.0))
+                                        : make_double2(0.0, 0.0);
+                ur = fma(-a.x, dr, fma(a.y, di, rr));
+                ui = fma(-a.x, di, fma(-a.y, dr, ri));
+            }
             const double2 iw = wa;
             wa = wb;
             if (j + 2 < N) wb = W[(int64_t)(j + 2) * nE_pad];
@@ -183,6 +193,7 @@ __global__ void k_ed_solve(const GroupDesc* __restrict__ groups, const ClassDesc
             }
         }
         s = F.add(f2d_int(sh), F.add(f2d_int(sl), s));
+        if (scheme == 0) s *= 4.0 / (inv_dx2 * inv_dx2);   // 1 / a^2
         if (k < nE) P_out[inst * (int64_t)nE + k] = (eps / 3.14159265358979323846) * s * C.dx;
     }
 }
@@ -216,7 +227,17 @@ cudaError_t launch_ionisation(const double* d_P, int64_t n_inst, int nE, const d
     return cudaGetLastError();
 }
 
-int64_t energy_distribution_scratch_elems(int sm_count, int n_max) { return (int64_t)sm_count * 8 * kLanes * n_max; }
+// Warps per SM: a warp's two dependent sweeps leave the FP64 pipe idle for half of the time at 8 warps; 16
+// while their scratch stays below 8 GB.
+static int solve_warps(int sm_count, int n_max)
+{
+    return (int64_t)sm_count * 16 * kLanes * n_max * (int64_t)sizeof(double2) <= (int64_t(8) << 30) ? 16 : 8;
+}
+
+int64_t energy_distribution_scratch_elems(int sm_count, int n_max)
+{
+    return (int64_t)sm_count * solve_warps(sm_count, n_max) * kLanes * n_max;
+}
 
 cudaError_t launch_energy_distribution(int mixed, const GroupDesc* d_groups, const ClassDesc* d_cls, int n_cls,
                                        const double* d_tab, const int64_t* d_slot_group, const int64_t* d_slot_inst,
@@ -232,17 +253,15 @@ cudaError_t launch_energy_distribution(int mixed, const GroupDesc* d_groups, con
     k_ed_pivots<<<pg, 128, 0, st>>>(d_cls, n_cls, d_tab, d_E_grid, nE, nE_pad, eps, scheme, pivW, pivC, d_piv_off);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const int blocks = sm_count;   // 8 warps per block: the scratch holds sm_count * 8 warps
+    const int blocks = sm_count * (solve_warps(sm_count, n_max) / 8);   // of 8 warps, as the scratch holds
+    auto solve = [&](auto kernel, auto psi) {
+        kernel<<<blocks, 256, 0, st>>>(d_groups, d_cls, d_tab, d_slot_group, d_slot_inst, n_slots, psi, d_E_grid, nE, nE_pad, eps,
+                                       pivW, pivC, d_piv_off, static_cast<double2*>(d_scratch), n_max, P_out);
+    };
     if (mixed)
-        k_ed_solve<float2><<<blocks, 256, 0, st>>>(d_groups, d_cls, d_tab, d_slot_group, d_slot_inst, n_slots,
-                                                   static_cast<const float2*>(d_psi), d_E_grid, nE, nE_pad, eps, scheme,
-                                                   pivW, pivC, d_piv_off, static_cast<double2*>(d_scratch), n_max,
-                                                   P_out);
+        solve(scheme == 0 ? k_ed_solve<float2, 0> : k_ed_solve<float2, 1>, static_cast<const float2*>(d_psi));
     else
-        k_ed_solve<double2><<<blocks, 256, 0, st>>>(d_groups, d_cls, d_tab, d_slot_group, d_slot_inst, n_slots,
-                                                    static_cast<const double2*>(d_psi), d_E_grid, nE, nE_pad, eps,
-                                                    scheme, pivW, pivC, d_piv_off, static_cast<double2*>(d_scratch),
-                                                    n_max, P_out);
+        solve(scheme == 0 ? k_ed_solve<double2, 0> : k_ed_solve<double2, 1>, static_cast<const double2*>(d_psi));
     return cudaGetLastError();
 }
 
