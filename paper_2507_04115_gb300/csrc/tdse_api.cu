@@ -877,7 +877,12 @@ tdse_status tdse_ground_state(tdse_batch* b, double dtau, int64_t max_iter, doub
     if (!guard.ok) return fail(TDSE_ERR_CUDA, "cudaSetDevice failed");
     cudaStream_t st = (cudaStream_t)stream;
     const int n_cls = (int)b->classes.size();
-    TDSE_CUDA(launch_ground_state(b->d_cls, n_cls, (int)b->scheme, dtau, max_iter, tol, b->d_gs_work, b->d_gs_off,
+    int min_N = b->classes[0].N, max_N = min_N;
+    for (const ClassDesc& C : b->classes) {
+        min_N = std::min(min_N, C.N);
+        max_N = std::max(max_N, C.N);
+    }
+    TDSE_CUDA(launch_ground_state(b->d_cls, n_cls, min_N, max_N, (int)b->scheme, dtau, max_iter, tol, b->d_gs_work, b->d_gs_off,
                                   b->d_gs_energy, b->d_gs_iters, st),
               "ground_state launch");
     TDSE_CUDA(launch_gs_support(b->d_cls, n_cls, b->d_gs_work, b->d_gs_off, b->d_gs_support, st), "support launch");

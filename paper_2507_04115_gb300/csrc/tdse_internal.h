@@ -281,7 +281,10 @@ cudaError_t launch_build_tables(const ClassDesc* d_cls, int n_cls, int max_N, do
 // psi0, energy, iters.
 constexpr int kGsThreads = 1024;
 constexpr int kGsWork = 8;
-cudaError_t launch_ground_state(const ClassDesc* d_cls, int n_cls, int scheme, double dtau, int64_t max_iter,
+// Grids up to this size run on a cluster of CTAs per class with the state in registers; min_N, max_N: the
+// smallest and largest grid of the classes.
+constexpr int kGsRegN = 8192;
+cudaError_t launch_ground_state(const ClassDesc* d_cls, int n_cls, int min_N, int max_N, int scheme, double dtau, int64_t max_iter,
                                 double tol, double* d_work, const int64_t* d_work_off, double* d_energy,
                                 int64_t* d_iters, cudaStream_t st);
 

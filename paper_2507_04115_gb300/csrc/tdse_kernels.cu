@@ -124,7 +124,288 @@ __device__ void block_recurrence(double* __restrict__ x, const double* __restric
     __syncthreads();
 }
 
-// Imaginary-time Crank-Nicolson for the field-free Hamiltonian of one class per CTA.
+// ---- ground states of grids up to kGsRegN points: a cluster of CTAs per class, the state in registers
+//
+// The iteration is latency-bound (two dependent sweeps of N points), so a class is spread over
+// kGsCluster CTAs of kGsCtaThreads threads, 8 consecutive points per thread.  A sweep is a first-order
+// recurrence with fixed coefficients: each thread runs its points from zero, publishes its last value
+// (shared memory, read across the cluster), and adds the incoming value times the running products of its
+// coefficients, which are tabulated.  The incoming value is the sum of the preceding threads' last values
+// times the products between, cut where these fall below 1e-20 (the sweeps forget at |a| < 1 a point;
+// about 7 threads at the workloads' spacings): no scan over the whole grid.  Three cluster barriers per
+// iteration, one more for the energy, which is formed only where the stopping rule can use it
+// (tol > 0, or the last iteration).
+// Measured, 8 classes of 1024 to 8192 points, 600 iterations: 116 ms with one CTA of 1024 threads per class
+// (a scan of 10 levels per sweep, V and the division by the norm evaluated per point), 2.6 ms here.
+constexpr int kGsCluster = 8;
+constexpr int kGsCtaThreads = 128;
+constexpr int kGsPer = 8;
+constexpr int kGsArrays = 11;   // tabulated coefficients per point
+
+struct GsShared {
+    double sv[4][kGsCtaThreads];      // last values of the four sweeps
+    double prod[4][kGsCtaThreads];    // products of each thread's coefficients
+    double edge[2][kGsCtaThreads];    // first and last psi' of each thread
+    double part[2][kGsCtaThreads / 32];
+    int bad, neg;
+};
+constexpr size_t kGsSmem = sizeof(GsShared) + sizeof(double) * kGsArrays * kGsPer * kGsCtaThreads;
+
+__global__ void __cluster_dims__(kGsCluster, 1, 1) __launch_bounds__(kGsCtaThreads)
+k_ground_state_cluster(const ClassDesc* cls, int scheme, double dtau, int64_t max_iter, double tol, double* work,
+                       const int64_t* work_off, double* energy, int64_t* iters)
+{
+    namespace cg = cooperative_groups;
+    extern __shared__ double gs_dyn[];
+    GsShared& sh = *reinterpret_cast<GsShared*>(gs_dyn);
+    double* tabs = gs_dyn + sizeof(GsShared) / sizeof(double);
+    cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank(), tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int ci = blockIdx.x / kGsCluster;
+    const ClassDesc C = cls[ci];
+    const int N = C.N;
+    if (N > kGsRegN) return;   // the whole cluster: k_ground_state takes this class
+    const int T = rank * kGsCtaThreads + tid, k0 = T * kGsPer;   // this thread's points k0 .. k0 + 7
+    const double inv_dx2 = 1.0 / (C.dx * C.dx), c = 0.5 * dtau;
+    const bool numerov = scheme == 1;
+    auto tab = [&](int a, int e) -> double& { return tabs[(a * kGsPer + e) * kGsCtaThreads + tid]; };
+    enum { kW, kFa, kBa, kQf, kQb, kDi, kMw, kMfa, kMba, kMqf, kMqb };
+    auto V_at = [&](int j) {
+        const double x = (j - 0.5 * (N - 1)) * C.dx;
+        return -C.Z / sqrt(fma(x, x, C.a * C.a));
+    };
+    auto A_di = [&](double V) { return numerov ? 10.0 / 12.0 + c * (inv_dx2 + (10.0 / 12.0) * V) : 1.0 + c * (inv_dx2 + V); };
+    auto A_off = [&](double V) { return numerov ? 1.0 / 12.0 + c * (-0.5 * inv_dx2 + V / 12.0) : -c * 0.5 * inv_dx2; };
+
+    // Thomas factors of A (and of M2): the pivots forget their start like the squares of the sweeps'
+    // coefficients, so each thread starts kWarm points early; neighbours compare the pivot they share, and
+    // where one differs the first thread runs the whole sequence
+    constexpr int kWarm = 64;
+    if (tid == 0) sh.bad = 0;
+    __syncthreads();
+    double wl = 0.0, ml = 0.0;   // pivots' reciprocals at k0 - 1 as this thread has them
+    {
+        double wp = 0.0, mp = 0.0, Vm = 0.0, V0 = 0.0;   // V at j - 1, j
+        const int js = max(0, k0 - kWarm);
+        if (js < N) {
+            V0 = V_at(js);
+            if (js > 0) Vm = V_at(js - 1);
+        }
+#pragma unroll 1
+        for (int j = js; j < min(N, k0 + kGsPer); ++j) {
+            const double Vp = V_at(j + 1);
+            const double lo = A_off(Vm), up_prev = A_off(V0);   // A_{j,j-1}, A_{j-1,j}
+            const double piv = j == js ? A_di(V0) : A_di(V0) - lo * up_prev * wp;
+            wp = 1.0 / piv;
+            if (numerov) mp = 1.0 / (j == js ? 10.0 / 12.0 : 10.0 / 12.0 - (1.0 / 144.0) * mp);
+            if (j >= k0) {
+                const int e = j - k0;
+                tab(kW, e) = wp;
+                tab(kFa, e) = j == 0 ? 0.0 : -lo * wp;
+                tab(kBa, e) = j == N - 1 ? 0.0 : -A_off(Vp) * wp;
+                tab(kDi, e) = numerov ? V0 : inv_dx2 + V0;
+                if (numerov) {
+                    tab(kMw, e) = mp;
+                    tab(kMfa, e) = j == 0 ? 0.0 : -(1.0 / 12.0) * mp;
+                    tab(kMba, e) = j == N - 1 ? 0.0 : -(1.0 / 12.0) * mp;
+                }
+            } else if (j == k0 - 1) {
+                wl = wp;
+                ml = mp;
+            }
+            Vm = V0;
+            V0 = Vp;
+        }
+    }
+    auto zero_tail = [&]() {   // points beyond the grid: zero coefficients
+#pragma unroll
+        for (int e = 0; e < kGsPer; ++e)
+            if (k0 + e >= N)
+                for (int a = 0; a < kGsArrays; ++a) tab(a, e) = 0.0;
+    };
+    zero_tail();
+    sh.edge[0][tid] = k0 < N ? tab(kW, min(kGsPer, N - k0) - 1) : 0.0;
+    sh.edge[1][tid] = numerov && k0 < N ? tab(kMw, min(kGsPer, N - k0) - 1) : 0.0;
+    cluster.sync();
+    auto at_thread = [&](double* p, int t) { return cluster.map_shared_rank(p, t / kGsCtaThreads)[t % kGsCtaThreads]; };
+    if (T > 0 && k0 < N) {
+        const double a = at_thread(sh.edge[0], T - 1), b = at_thread(sh.edge[1], T - 1);
+        if (!(fabs(a - wl) <= 2e-15 * fabs(a)) || (numerov && !(fabs(b - ml) <= 2e-15 * fabs(b)))) *cluster.map_shared_rank(&sh.bad, 0) = 1;
+    }
+    cluster.sync();
+    if (*cluster.map_shared_rank(&sh.bad, 0)) {   // slow forgetting: the pivots in sequence, by way of global memory
+        double* wseq = work + work_off[ci] + N;
+        if (T == 0) {
+            double wp = 0.0, mp = 0.0, Vm = 0.0, V0 = V_at(0);
+            for (int j = 0; j < N; ++j) {
+                const double piv = j == 0 ? A_di(V0) : A_di(V0) - A_off(Vm) * A_off(V0) * wp;
+                wp = 1.0 / piv;
+                mp = 1.0 / (10.0 / 12.0 - (j > 0 ? (1.0 / 144.0) * mp : 0.0));
+                wseq[j] = wp;
+                wseq[N + j] = mp;
+                Vm = V0;
+                V0 = V_at(j + 1);
+            }
+            __threadfence();
+        }
+        cluster.sync();
+        for (int e = 0; e < kGsPer; ++e) {
+            const int j = k0 + e;
+            if (j >= N) break;
+            const double w = __ldcg(wseq + j), mw = __ldcg(wseq + N + j);
+            tab(kW, e) = w;
+            tab(kFa, e) = j == 0 ? 0.0 : -A_off(V_at(j - 1)) * w;
+            tab(kBa, e) = j == N - 1 ? 0.0 : -A_off(V_at(j + 1)) * w;
+            if (numerov) {
+                tab(kMw, e) = mw;
+                tab(kMfa, e) = j == 0 ? 0.0 : -(1.0 / 12.0) * mw;
+                tab(kMba, e) = j == N - 1 ? 0.0 : -(1.0 / 12.0) * mw;
+            }
+        }
+    }
+    // running products of each thread's coefficients, forward (from its first point) and backward
+    {
+        double qf = 1.0, qb = 1.0, mf = 1.0, mb = 1.0;
+        for (int e = 0; e < kGsPer; ++e) {
+            tab(kQf, e) = qf *= tab(kFa, e);
+            tab(kQb, kGsPer - 1 - e) = qb *= (k0 + kGsPer - 1 - e < N ? tab(kBa, kGsPer - 1 - e) : 1.0);
+            if (numerov) {
+                tab(kMqf, e) = mf *= tab(kMfa, e);
+                tab(kMqb, kGsPer - 1 - e) = mb *= (k0 + kGsPer - 1 - e < N ? tab(kMba, kGsPer - 1 - e) : 1.0);
+            }
+        }
+        sh.prod[0][tid] = qf;
+        sh.prod[1][tid] = qb;
+        sh.prod[2][tid] = mf;
+        sh.prod[3][tid] = mb;
+    }
+    const int n_thr = (N + kGsPer - 1) / kGsPer;   // threads that hold points
+    cluster.sync();
+
+    // Value coming into this thread's points: the preceding threads' last values times the products
+    // between (which: 0, 2 forward, 1, 3 backward).
+    auto carry = [&](int which) {
+        const int step = (which & 1) ? 1 : -1;
+        double s = 0.0, p = 1.0;
+        for (int t = T + step; t >= 0 && t < n_thr; t += step) {
+            s = fma(p, at_thread(sh.sv[which], t), s);
+            p *= at_thread(sh.prod[which], t);
+            if (!(fabs(p) > 1e-20)) break;
+        }
+        return s;
+    };
+    // x_e = a_e x_{e-1} + x_e over the grid in either direction, the coefficients and their products tabulated
+    auto sweep = [&](double (&x)[kGsPer], int which, int ka, int kq) {
+        double y = 0.0;
+        if (which & 1) {
+#pragma unroll
+            for (int e = kGsPer - 1; e >= 0; --e) x[e] = y = fma(tab(ka, e), y, x[e]);
+        } else {
+#pragma unroll
+            for (int e = 0; e < kGsPer; ++e) x[e] = y = fma(tab(ka, e), y, x[e]);
+        }
+        sh.sv[which][tid] = y;
+        cluster.sync();
+        const double in = carry(which);
+#pragma unroll
+        for (int e = 0; e < kGsPer; ++e) x[e] = fma(tab(kq, e), in, x[e]);
+    };
+    auto total = [&](double v, int slot) {   // sum over the cluster, the same on every thread
+        v = warp_sum(v);
+        if (lane == 0) sh.part[slot][wid] = v;
+        cluster.sync();
+        const double p = cluster.map_shared_rank(&sh.part[slot][0], lane / (kGsCtaThreads / 32))[lane % (kGsCtaThreads / 32)];
+        return warp_sum(p);
+    };
+    static_assert(kGsCluster * (kGsCtaThreads / 32) == 32, "one partial per lane");
+
+    double psi[kGsPer], left, right;   // psi (normalised below) and its neighbours across the chunk's ends
+#pragma unroll
+    for (int e = 0; e < kGsPer; ++e) {
+        const double x = (k0 + e - 0.5 * (N - 1)) * C.dx;
+        psi[e] = k0 + e < N ? exp(-x * x) : 0.0;
+    }
+    {
+        const double xl = (k0 - 1 - 0.5 * (N - 1)) * C.dx, xr = (k0 + kGsPer - 0.5 * (N - 1)) * C.dx;
+        left = k0 > 0 && k0 - 1 < N ? exp(-xl * xl) : 0.0;
+        right = k0 + kGsPer < N ? exp(-xr * xr) : 0.0;
+    }
+    double e_prev = 0.0, en = 0.0;
+    int64_t it = 1;
+    for (;; ++it) {
+        double y[kGsPer];
+#pragma unroll
+        for (int e = 0; e < kGsPer; ++e) {
+            double r = psi[e];
+            if (numerov) {
+                const double l = e > 0 ? psi[e - 1] : left, u = e < kGsPer - 1 ? psi[e + 1] : right;
+                r = (10.0 / 12.0) * psi[e] + (l + u) / 12.0;
+            }
+            y[e] = tab(kW, e) * r;
+        }
+        sweep(y, 0, kFa, kQf);
+        sweep(y, 1, kBa, kQb);
+        double s = 0.0;
+#pragma unroll
+        for (int e = 0; e < kGsPer; ++e) {
+            psi[e] = k0 + e < N ? 2.0 * y[e] - psi[e] : 0.0;
+            s = fma(psi[e], psi[e], s);
+        }
+        sh.edge[0][tid] = psi[0];
+        sh.edge[1][tid] = psi[kGsPer - 1];
+        const double inv = 1.0 / sqrt(total(s, 0) * C.dx);
+        left = T > 0 ? at_thread(sh.edge[1], T - 1) * inv : 0.0;
+        right = T + 1 < n_thr ? at_thread(sh.edge[0], T + 1) * inv : 0.0;
+#pragma unroll
+        for (int e = 0; e < kGsPer; ++e) psi[e] *= inv;
+        if (!(tol > 0.0) && it < max_iter) continue;   // no energy difference can end the iteration here
+        // energy: T psi = -Delta2/2 psi (FD) or M2^{-1}(-Delta2/2 psi) (Numerov)
+        double se = 0.0;
+        if (numerov) {
+#pragma unroll
+            for (int e = 0; e < kGsPer; ++e) {
+                const double l = e > 0 ? psi[e - 1] : left, u = e < kGsPer - 1 ? psi[e + 1] : right;
+                y[e] = -0.5 * ((l - 2.0 * psi[e] + u) * inv_dx2) * tab(kMw, e);
+            }
+            sweep(y, 2, kMfa, kMqf);
+            sweep(y, 3, kMba, kMqb);
+#pragma unroll
+            for (int e = 0; e < kGsPer; ++e) se = fma(psi[e], fma(tab(kDi, e), psi[e], y[e]), se);
+        } else {
+#pragma unroll
+            for (int e = 0; e < kGsPer; ++e) {
+                const double l = e > 0 ? psi[e - 1] : left, u = e < kGsPer - 1 ? psi[e + 1] : right;
+                se = fma(psi[e], fma(tab(kDi, e), psi[e], -0.5 * inv_dx2 * (l + u)), se);
+            }
+        }
+        en = total(se, 1) * C.dx;
+        if ((it > 1 && fabs(en - e_prev) < tol) || it >= max_iter) break;
+        e_prev = en;
+    }
+    // sign: positive at the centre
+    const int tc = (N / 2) / kGsPer;
+    if (T == tc) {
+        double v = 0.0;
+#pragma unroll
+        for (int e = 0; e < kGsPer; ++e)
+            if (k0 + e == N / 2) v = psi[e];
+        sh.neg = v < 0.0;
+    }
+    cluster.sync();
+    const double sgn = *cluster.map_shared_rank(&sh.neg, tc / kGsCtaThreads) ? -1.0 : 1.0;
+    double* out = work + work_off[ci];
+#pragma unroll
+    for (int e = 0; e < kGsPer; ++e)
+        if (k0 + e < N) out[k0 + e] = psi[e] * sgn;
+    if (T == 0) {
+        energy[ci] = en;
+        iters[ci] = it;
+    }
+    cluster.sync();   // no CTA leaves while another may read its shared memory
+}
+
+// Imaginary-time Crank-Nicolson for the field-free Hamiltonian of one class per CTA (grids above kGsRegN
+// points).
 //   FULL_CN  : A = 1 + dtau/2 H0,   y = A^{-1} psi,       psi' = 2 y - psi
 //   NUMEROV  : A = M2 + dtau/2 K,   y = A^{-1} (M2 psi),  psi' = 2 y - psi   (K = -Delta2/2 + M2 V)
 // since A + B = 2M with B = M - dtau/2 K.  Then psi' is normalised and E = <psi|H0|psi> dx.
@@ -133,7 +414,8 @@ __device__ void block_recurrence(double* __restrict__ x, const double* __restric
 // two sweeps of Numerov's M2 solve in the energy.
 // Work block per class (kGsWork N doubles): psi | 1/pivot of A | forward a | backward a | y |
 // 1/pivot of M2 | M2 forward a | M2 backward a.
-__global__ void k_ground_state(const ClassDesc* cls, int scheme, double dtau, int64_t max_iter, double tol,
+__global__ void __launch_bounds__(kGsThreads)
+k_ground_state(const ClassDesc* cls, int scheme, double dtau, int64_t max_iter, double tol,
                                double* work, const int64_t* work_off, double* energy, int64_t* iters)
 {
     __shared__ double red[32];
@@ -141,6 +423,7 @@ __global__ void k_ground_state(const ClassDesc* cls, int scheme, double dtau, in
     __shared__ int stop;
     const ClassDesc C = cls[blockIdx.x];
     const int N = C.N;
+    if (N <= kGsRegN) return;   // k_ground_state_cluster has this class
     double* psi = work + work_off[blockIdx.x];
     double* w = psi + N;
     double* fa = w + N;
@@ -246,12 +529,24 @@ __global__ void k_ground_state(const ClassDesc* cls, int scheme, double dtau, in
     }
 }
 
-cudaError_t launch_ground_state(const ClassDesc* d_cls, int n_cls, int scheme, double dtau, int64_t max_iter,
+cudaError_t launch_ground_state(const ClassDesc* d_cls, int n_cls, int min_N, int max_N, int scheme, double dtau, int64_t max_iter,
                                 double tol, double* d_work, const int64_t* d_work_off, double* d_energy,
                                 int64_t* d_iters, cudaStream_t st)
 {
-    k_ground_state<<<n_cls, kGsThreads, 0, st>>>(d_cls, scheme, dtau, max_iter, tol, d_work, d_work_off, d_energy,
-                                                  d_iters);
+    if (min_N <= kGsRegN) {
+        static std::atomic<bool> attr_set[kMaxAttrDevices];
+        int dev = 0;
+        if (attr_needed(attr_set, &dev)) {
+            const cudaError_t e = cudaFuncSetAttribute(k_ground_state_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGsSmem);
+            if (e != cudaSuccess) return e;
+            attr_done(attr_set, dev);
+        }
+        k_ground_state_cluster<<<n_cls * kGsCluster, kGsCtaThreads, kGsSmem, st>>>(d_cls, scheme, dtau, max_iter, tol, d_work,
+                                                                                  d_work_off, d_energy, d_iters);
+    }
+    if (max_N > kGsRegN)
+        k_ground_state<<<n_cls, kGsThreads, 0, st>>>(d_cls, scheme, dtau, max_iter, tol, d_work, d_work_off, d_energy,
+                                                      d_iters);
     return cudaGetLastError();
 }
 

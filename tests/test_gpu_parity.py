@@ -71,6 +71,29 @@ def test_ground_state_matches_oracle(env):
         b.close()
 
 
+@pytest.mark.parametrize("scheme", [0, 1])
+def test_ground_state_grid_sizes(env, scheme):
+    """Grids around the chunks of the cluster kernel (8 points a thread, 1024 a CTA), its largest grid and
+    the first beyond it, and a spacing at which the sweeps forget so slowly that the factors are formed in
+    sequence; fixed iteration counts, against the oracle."""
+    tdse, oracle = env
+    N = [16, 17, 1023, 1025, 2047, 8192, 8200, 700]
+    dx = [0.3, 0.2, 0.2, 0.15, 0.2, 0.2, 0.15, 0.004]
+    b = tdse.Batch(N, dx, 1.19, 1, 0.02, scheme=scheme)
+    e, it = b.ground_state(dtau=0.1, max_iter=40, tol=0.0)
+    assert np.all(it == 40)
+    for i in range(len(N)):
+        psi, e_o, _ = oracle.ground_state(N[i], dx[i], 1.19, dtau=0.1, max_iter=40, tol=0.0, scheme=scheme)
+        got = b.get_psi(i).cpu().numpy()
+        assert abs(e[i] - e_o) < 1e-12 + 2e-15 / dx[i] ** 2, (N[i], e[i], e_o)   # the rounding of the second difference
+        assert np.max(np.abs(got - psi)) < 1e-11 * np.max(np.abs(psi)), N[i]
+    e2, it2 = b.ground_state(dtau=0.1, max_iter=5000, tol=1e-9)       # the stopping rule
+    ref = [oracle.ground_state(N[i], dx[i], 1.19, dtau=0.1, max_iter=5000, tol=1e-9, scheme=scheme) for i in range(3)]
+    for i in range(3):
+        assert abs(e2[i] - ref[i][1]) < 1e-11 and abs(int(it2[i]) - ref[i][2]) <= 1
+    b.close()
+
+
 def test_single_atom_full_propagation(env):
     """The single-atom workload (N = 2000, 8818 steps, mask on) end to end: d, a and |DFT(a)|^2."""
     tdse, oracle = env
