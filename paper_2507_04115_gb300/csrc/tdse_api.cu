@@ -201,9 +201,10 @@ void free_device(tdse_batch* b)
 //   A_{j,j+1} = 1/12 + i h (-1/(2dx^2) + V_{j+1}/12);
 // Thomas from j = 0: pivot_j = A_jj - A_{j,j-1} C_{j-1}, W_j = 1/pivot_j, L_j = A_{j,j-1} W_j,
 // C_j = A_{j,j+1} W_j.  Writes (W_j/12, L_j, C_j) as double pairs and float pairs into the host
-// images of the nw/nl/nc/nf tables and returns max(|L|, |C|).
-double numerov_factors(const ClassDesc& C, double dt, std::vector<double>& nw, std::vector<double>& nl,
-                       std::vector<double>& nc, std::vector<float>& nf)
+// images of the nw/nl/nc/nf tables and returns max(|L|, |C|); with C.fix.num also the fixed-point factors,
+// clearing it where they leave its range (|L|, |C| <= 0.35, |W|/12 <= 0.115: digit products in 63 bits).
+double numerov_factors(ClassDesc& C, double dt, std::vector<double>& nw, std::vector<double>& nl,
+                       std::vector<double>& nc, std::vector<float>& nf, std::vector<int32_t>& fix)
 {
     using cd = std::complex<double>;
     const int N = C.N;
@@ -217,7 +218,7 @@ double numerov_factors(const ClassDesc& C, double dt, std::vector<double>& nw, s
     nl.assign(2 * (size_t)N, 0.0);
     nc.assign(2 * (size_t)N, 0.0);
     nf.assign(6 * (size_t)N, 0.0f);
-    double rho = 0.0;
+    double rho = 0.0, w_max = 0.0;
     cd cprev(0.0, 0.0);
     for (int j = 0; j < N; ++j) {
         const cd lo = j > 0 ? cd(1.0 / 12.0, h * (-0.5 * inv + V[j - 1] / 12.0)) : cd(0.0, 0.0);
@@ -241,7 +242,26 @@ double numerov_factors(const ClassDesc& C, double dt, std::vector<double>& nw, s
         nf[6 * j + 4] = (float)Cj.real();
         nf[6 * j + 5] = (float)Cj.imag();
         rho = std::max(rho, std::max(std::abs(L), std::abs(Cj)));
+        w_max = std::max(w_max, std::abs(W12));
         cprev = Cj;
+    }
+    fix.clear();
+    if (!(rho <= 0.35 && w_max <= 0.115)) C.fix.num = 0;
+    if (C.fix.num) {
+        fix.reserve(12 * (size_t)N);
+        auto put = [&](double v, int k) {
+            const Digits d = digits(std::llrint(std::ldexp(v, k)));
+            fix.push_back(d.h);
+            fix.push_back(d.l);
+        };
+        for (int j = 0; j < N; ++j) {
+            put(nw[2 * j], 65);
+            put(nw[2 * j + 1], 65);
+            put(-nl[2 * j], 64);
+            put(-nl[2 * j + 1], 64);
+            put(-nc[2 * j], 64);
+            put(-nc[2 * j + 1], 64);
+        }
     }
     return rho;
 }
@@ -272,6 +292,8 @@ void build_classes(tdse_batch* b, const tdse_instance* inst_host, int64_t n_inst
             C.one = 1.0;
             C.nzero = -0.0;
             C.fix = class_fix(C, dt);
+            // NUMEROV_SPLIT: settled when the factors are known (numerov_factors); N as for FULL_CN
+            C.fix.num = b->scheme == TDSE_NUMEROV_SPLIT && b->precision == TDSE_FP64 && I.N <= 32768 && C.fix.kv <= 60;
             b->classes.push_back(C);
         } else {
             c = it->second;
@@ -465,8 +487,9 @@ tdse_status build_groups(tdse_batch* b)
 // Groups of a batch that the fixed-point sweep serves.
 bool on_fix_path(const tdse_batch* b, const ClassDesc& C)
 {
-    return b->precision == TDSE_FP64 && b->scheme == TDSE_FULL_CN && C.fix.ok;
+    return b->precision == TDSE_FP64 && (b->scheme == TDSE_FULL_CN ? C.fix.ok : C.fix.num);
 }
+double fix_lead(const tdse_batch* b) { return b->scheme == TDSE_FULL_CN ? kLeadFullCn : kLeadNumerov; }
 
 // Warps, halo, segment length and priority of every group by the FP64 pipe's rules (or, with `fix`, by
 // those of the fixed-point sweep at per_sm CTAs per SM where a class has that form); returns the rows of a
@@ -483,12 +506,12 @@ int shape_groups(const tdse_batch* b, std::vector<GroupDesc>& groups, bool fix, 
         int K = class_halo(b, C);
         const bool fx = fix && on_fix_path(b, C);
         const int cap = fix && b->warps_override <= 0 ? std::min(most, most_fix) : most;
-        const int P = fx ? fix_warps(C.N, K, L, most_fix, per_sm) : group_warps(C.N, K, L, cap);
+        const int P = fx ? fix_warps(C.N, K, L, most_fix, per_sm, fix_lead(b)) : group_warps(C.N, K, L, cap);
         if (P == 1 && L == 1) K = 0;   // one exact segment
         G.P = P;
         G.K = K;
         G.m = group_segment_length(G.N, P, L);
-        G.w = std::max(1, (int)std::lround((fx ? fix_step_cost(C.N, K, L, P, P * per_sm) : group_step_cost(C.N, K, L, cap)) / 64.0));
+        G.w = std::max(1, (int)std::lround((fx ? fix_step_cost(C.N, K, L, P, P * per_sm, fix_lead(b)) : group_step_cost(C.N, K, L, cap)) / 64.0));
         *widest = std::max(*widest, fx ? P : cap);
         // a sweep covers its segment and a halo on each side (m + 2K rows; the 32-wide propagation
         // clips it at the walls); a single exact segment covers the N points
@@ -512,7 +535,7 @@ tdse_status build_plan(tdse_batch* b)
         std::vector<FixGroup> g;
         for (const GroupDesc& G : b->groups)
             g.push_back({G.N, class_halo(b, b->classes[G.cls]), kLanes / G.I, (double)std::max<int64_t>(G.nt_max, 1)});
-        want = fix_ctas_per_sm(g, b->sm_count);
+        want = fix_ctas_per_sm(g, b->sm_count, fix_lead(b));
     }
     const int shape_per_sm = want >= 4 ? 4 : (want >= 2 ? 2 : 1);
     b->rows = shape_groups(b, b->groups, fix, shape_per_sm, &b->warps);
@@ -732,9 +755,12 @@ tdse_status tdse_batch_create(const tdse_instance* inst_host, int64_t n_inst, do
     if (scheme == TDSE_NUMEROV_SPLIT) {
         std::vector<double> nw, nl, nc;
         std::vector<float> nf;
+        std::vector<int32_t> fix;
         for (auto& C : b->classes) {
-            C.rho = numerov_factors(C, dt, nw, nl, nc, nf);
-            if ((e = cudaMemcpy(b->d_tab + tab_nw(C), nw.data(), sizeof(double) * nw.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
+            C.rho = numerov_factors(C, dt, nw, nl, nc, nf, fix);
+            if ((!fix.empty() &&
+                 (e = cudaMemcpy(b->d_tab + tab_fnw(C), fix.data(), sizeof(int32_t) * fix.size(), cudaMemcpyHostToDevice)) != cudaSuccess) ||
+                (e = cudaMemcpy(b->d_tab + tab_nw(C), nw.data(), sizeof(double) * nw.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
                 (e = cudaMemcpy(b->d_tab + tab_nl(C), nl.data(), sizeof(double) * nl.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
                 (e = cudaMemcpy(b->d_tab + tab_nc(C), nc.data(), sizeof(double) * nc.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
                 (e = cudaMemcpy(b->d_tab + tab_nf(C), nf.data(), sizeof(float) * nf.size(), cudaMemcpyHostToDevice)) != cudaSuccess)
@@ -801,7 +827,8 @@ tdse_status tdse_model_layout(const tdse_instance* inst_host, int64_t n_inst, do
     if (scheme == TDSE_NUMEROV_SPLIT) {
         std::vector<double> nw, nl, nc;
         std::vector<float> nf;
-        for (auto& C : tmp.classes) C.rho = numerov_factors(C, dt, nw, nl, nc, nf);
+        std::vector<int32_t> fix;
+        for (auto& C : tmp.classes) C.rho = numerov_factors(C, dt, nw, nl, nc, nf, fix);
     }
     std::vector<int64_t> count(tmp.classes.size(), 0);
     for (int64_t i = 0; i < n_inst; ++i) ++count[tmp.inst_class[i]];

@@ -45,7 +45,8 @@ struct Digits {
 };
 
 struct FixClass {
-    int32_t ok;             // the class has a fixed-point form (0: the FP64 sweep)
+    int32_t ok;             // FULL_CN has a fixed-point form (0: the FP64 sweep)
+    int32_t num;            // NUMEROV_SPLIT has one
     int32_t top, xk, kv;
     int32_t ci;             // 2/beta = ci + cf 2^-64
     Digits cf;
@@ -230,6 +231,8 @@ inline int64_t pair_fix(double hi, double lo, int k) { return std::llrint(std::l
 inline FixClass fix_class(int N, double dx, double dt, double s0_max, double x_max, double dv_max)
 {
     FixClass f{};
+    f.kv = dv_max > 0.0 && std::isfinite(dv_max) ? std::max(-40, (int)std::ceil(std::log2(dv_max))) : 0;
+    f.v_scale = std::ldexp(1.0, f.kv - 61);
     const double beta = dt / (4.0 * dx * dx);
     // beta <= 0.35: gamma at 2^64 keeps its digit products in 63 bits; beta > 0.0715: Q < 16.  N: the sum
     // of (2j - N + 1) x low digit over a segment stays in 64 bits, and the rounding of one unit per
@@ -243,13 +246,11 @@ inline FixClass fix_class(int N, double dx, double dt, double s0_max, double x_m
     f.top = beta <= 0.25 ? 61 : 60;
     f.E_lim = 0.999 * (15.0 - s0_max) / x_max;   // |gamma| < 1 joins Q's components
     f.xk = (int)std::ceil(std::log2(x_max));
-    f.kv = dv_max > 0.0 ? std::max(-40, (int)std::ceil(std::log2(dv_max))) : 0;
     if (std::abs(f.xk) > 60 || f.kv > 60) return f;
     f.inv_b = pair_fix(ib, ib_lo, 58);
     f.ci = (int)std::lrint(2.0 * ib);
     f.cf = digits(pair_fix(2.0 * ib - f.ci, 2.0 * ib_lo, 63) * 2);
     f.e_scale = std::ldexp(1.0, 56 + f.xk);       // X E: 2^(61 - xk) 2^(56 + xk) 2^-59 = 2^58
-    f.v_scale = std::ldexp(1.0, f.kv - 61);
     f.ok = 1;
     return f;
 }

@@ -29,7 +29,8 @@ constexpr int kMaxSegments = 16;    // warps per CTA at most (512 threads)
 //   af[j]  = ab[j] rounded to float2                                      (float halo rows)
 //   xff[j] = (x_j, dV_j) as float pairs (hi, lo), hi = x rounded to float, lo = x - hi rounded
 //            to float: a float4 (x_hi, x_lo, dV_hi, dV_lo)
-//   fxp[j] = FixPoint, fob[j] = FixObs: the fixed-point sweep's tables (classes with fix.ok)
+//   fxp[j] = FixPoint, fob[j] = FixObs: the fixed-point sweeps' tables (classes with fix.ok or fix.num)
+//   fnw[j] = W_j/12 (2^65), -L_j, -C_j (2^64) as digits (re.h, re.l, im.h, im.l) (classes with fix.num)
 struct ClassDesc {
     int64_t tab_off;      // offset (in doubles) of the class block in the table buffer
     int32_t N;
@@ -74,7 +75,8 @@ __host__ __device__ inline int64_t tab_af(const ClassDesc& c) { return c.tab_off
 __host__ __device__ inline int64_t tab_xff(const ClassDesc& c) { return c.tab_off + 18 * tab_n(c.N); }
 __host__ __device__ inline int64_t tab_fxp(const ClassDesc& c) { return c.tab_off + 20 * tab_n(c.N); }
 __host__ __device__ inline int64_t tab_fob(const ClassDesc& c) { return c.tab_off + 22 * tab_n(c.N); }
-inline int64_t tab_doubles(const ClassDesc& c) { return (c.fix.ok ? 24 : 20) * tab_n(c.N); }
+__host__ __device__ inline int64_t tab_fnw(const ClassDesc& c) { return c.tab_off + 24 * tab_n(c.N); }
+inline int64_t tab_doubles(const ClassDesc& c) { return (c.fix.num ? 30 : (c.fix.ok ? 24 : 20)) * tab_n(c.N); }
 
 // ---- host-side planning rules shared by the allocating and the static entry points ----
 
@@ -137,19 +139,22 @@ inline double group_step_cost(int N, int K, int L, int warps)
 // other warps as far as they are, and everyone's instructions.  Measured, volume batch (K = 28, 160
 // steps): 120 ms at 8 warps, 104 at 12, 100 at 16, 113 with two CTAs of 8; one atom (K = 36, L = 32, 512
 // steps): 23.7 ms at 2 warps, 18.8 at 4, 20.9 at 8.
-inline double fix_step_cost(int N, int K, int L, int P, int W)
+// `lead`: whole rows' worth of a halo row, 1.3 there; 0.6 for NUMEROV_SPLIT (tdse_numerov_fix.cuh), whose
+// lead-ins run one sweep each.
+constexpr double kLeadFullCn = 1.3, kLeadNumerov = 0.6;
+inline double fix_step_cost(int N, int K, int L, int P, int W, double lead)
 {
     const int m = group_segment_length(N, P, L);
-    return 0.17 * (6.0 + std::max(W, 4)) * (m + 1.3 * (P * L > 1 ? K : 0));
+    return 0.17 * (6.0 + std::max(W, 4)) * (m + lead * (P * L > 1 ? K : 0));
 }
 // Warps carrying segments there when `per_sm` CTAs share an SM: the cheapest of those that group_warps
 // allows, segments of at least 4 points (a pass reads its own rows three ahead).
-inline int fix_warps(int N, int K, int L, int warps, int per_sm)
+inline int fix_warps(int N, int K, int L, int warps, int per_sm, double lead)
 {
     int best = 1;
     for (int P = 2; P <= group_warps(N, K, L, warps); ++P)
         if (group_segment_length(N, P, L) >= 4 &&
-            fix_step_cost(N, K, L, P, P * per_sm) < fix_step_cost(N, K, L, best, best * per_sm)) best = P;
+            fix_step_cost(N, K, L, P, P * per_sm, lead) < fix_step_cost(N, K, L, best, best * per_sm, lead)) best = P;
     return best;
 }
 
@@ -163,7 +168,7 @@ struct FixGroup {
     int N, K, L;
     double nt;
 };
-inline int fix_ctas_per_sm(const std::vector<FixGroup>& groups, int sm_count)
+inline int fix_ctas_per_sm(const std::vector<FixGroup>& groups, int sm_count, double lead)
 {
     double best_t = 0.0;
     int best = 1;
@@ -171,8 +176,8 @@ inline int fix_ctas_per_sm(const std::vector<FixGroup>& groups, int sm_count)
         double work = 0.0, longest = 0.0;
         const int share = (int)std::min<int64_t>(c, ((int64_t)groups.size() + sm_count - 1) / sm_count);
         for (const FixGroup& g : groups) {
-            const int P = fix_warps(g.N, g.K, g.L, kMaxSegments / c, c);
-            const double t = g.nt * fix_step_cost(g.N, g.K, g.L, P, P * share);
+            const int P = fix_warps(g.N, g.K, g.L, kMaxSegments / c, c, lead);
+            const double t = g.nt * fix_step_cost(g.N, g.K, g.L, P, P * share, lead);
             work += t / share;
             longest = std::max(longest, t);
         }

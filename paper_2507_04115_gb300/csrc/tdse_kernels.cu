@@ -61,10 +61,8 @@ __global__ void k_build_tables(const ClassDesc* cls, int n_cls, double dt, doubl
         const float xh = (float)x, vh = (float)dV;
         reinterpret_cast<float4*>(tab + tab_xff(C))[j] = make_float4(xh, (float)(x - (double)xh), vh, (float)(dV - (double)vh));
         tab[tab_vv(C) + j] = V;
-        if (C.fix.ok) {
-            reinterpret_cast<FixPoint*>(tab + tab_fxp(C))[j] = fix_point(C.fix, j, C.N, C.dx, V);
-            reinterpret_cast<FixObs*>(tab + tab_fob(C))[j] = fix_obs(C.fix, dV, m);
-        }
+        if (C.fix.ok) reinterpret_cast<FixPoint*>(tab + tab_fxp(C))[j] = fix_point(C.fix, j, C.N, C.dx, V);
+        if (C.fix.ok || C.fix.num) reinterpret_cast<FixObs*>(tab + tab_fob(C))[j] = fix_obs(C.fix, dV, m);
     }
 }
 

@@ -1,7 +1,7 @@
 // NUMEROV_SPLIT real-time propagation kernel of libtdse (sm_103a), FP64 and MIXED precision.  It
 // shares the lane-batched layout, the halo-segmented sweeps and the persistent group scheduler of
 // the FULL_CN kernel (see tdse_full_cn.cu).
-#include "tdse_sched.cuh"
+#include "tdse_numerov_fix.cuh"
 
 namespace tdse {
 
@@ -282,7 +282,15 @@ k_propagate_numerov(const GroupDesc* __restrict__ groups, int64_t n_groups, cons
         const int64_t n1 = min(n_end, n0 + slice);
         const double x0 = -0.5 * (N - 1) * dx;
 
-        if (G.I != kLanes) {
+        bool done = false;
+        if constexpr (!kMixed)
+            if (C.fix.num)
+                done = fix_numerov_slice(G, C, tab, ps, nt, row, slot, n0, n1, kslice == 0 && step_begin == 0, dt, E, d_out,
+                                         a_out, sample_base,
+                                         reinterpret_cast<int4*>(scratch_raw) + (int64_t)blockIdx.x * P * rows * (2 * kLanes),
+                                         red, status, jm_lo, jm_hi);
+        if (done) {
+        } else if (G.I != kLanes) {
             numerov_split_slice<kMixed>(G, C, F, ps, tW, tL, tC, tF, tab_xv2, tab_m, jm_lo, jm_hi, nt, row, slot, n0,
                                         n1, kslice == 0 && step_begin == 0, dt, E, d_out, a_out, sample_base, sc, red,
                                         status, kMixed ? tab_f4 : tab_xff4);

@@ -877,11 +877,14 @@ def test_lane_split_matches_32_wide(env):
             assert _rel(outs[lanes][1][sl], outs[1][1][sl]) < 1e-11, (lanes, i)
 
 
-@pytest.mark.parametrize("N,lanes,warps", [(2000, 32, 16), (401, 8, 2), (130, 32, 1), (96, 32, 16), (333, 1, 3)])
-def test_fixed_point_sweep_edges(env, N, lanes, warps):
-    """The fixed-point sweep where it can go wrong: segments shorter than the halo and shorter than the
-    four rows it needs (then the FP64 sweep runs), an odd grid, segments beyond the wall, instances that
-    end inside a slice, one-step chunks, and states of any norm (the scale is per instance)."""
+@pytest.mark.parametrize("scheme", [0, 1])
+@pytest.mark.parametrize("N,lanes,warps", [(2000, 32, 16), (2000, 32, 2), (401, 8, 2), (130, 32, 1), (96, 32, 16), (333, 1, 3),
+                                           (600, 2, 2)])
+def test_fixed_point_sweep_edges(env, N, lanes, warps, scheme):
+    """The fixed-point sweeps of both schemes where they can go wrong: segments shorter than the halo, of
+    one row, about as long as the halo and several times as long (FULL_CN has a form for either), odd grids,
+    segments beyond the wall, instances that end inside a slice, one-step chunks, and states of any norm
+    (the scale is per instance)."""
     tdse, oracle = env
     from paper_2507_04115_gb300 import inputs
     dx, dt, a = 0.2, 0.05, 1.19
@@ -890,7 +893,7 @@ def test_fixed_point_sweep_edges(env, N, lanes, warps):
     rows = [inputs.sin2_pulse(k, dt, 0.08, 0.3, 1.0, 0.4 * i) for i, k in enumerate(nt)]
     offs = np.concatenate([[0], np.cumsum(np.array(nt) + 1)])
     Et = _device_rows(rows, offs, torch.device("cuda", 0))
-    b = tdse.Batch([N] * 3, dx, a, nt, dt, row_offsets=offs, absorber=(5.0, 0.125), lanes_per_instance=lanes)
+    b = tdse.Batch([N] * 3, dx, a, nt, dt, row_offsets=offs, absorber=(5.0, 0.125), lanes_per_instance=lanes, scheme=scheme)
     b.set_launch(warps_per_cta=warps, slice_steps=9)
     b.ground_state(**GS_KW)
     psi0 = b.get_psi(0)
@@ -902,7 +905,7 @@ def test_fixed_point_sweep_edges(env, N, lanes, warps):
     m = oracle.mask(N, dx, 5.0, 0.125)
     p0 = psi0.cpu().numpy().real.copy()
     for i in range(3):
-        psi, d_o, a_o = oracle.propagate(p0, rows[i], dx, dt, a, mask_values=m)
+        psi, d_o, a_o = oracle.propagate(p0, rows[i], dx, dt, a, scheme=scheme, mask_values=m)
         sl = slice(offs[i], offs[i + 1])
         assert _rel(d[sl].cpu().numpy() / scale[i] ** 2, d_o) < RTOL_SERIES, i
         assert _rel(acc[sl].cpu().numpy() / scale[i] ** 2, a_o) < RTOL_SERIES, i
@@ -910,9 +913,10 @@ def test_fixed_point_sweep_edges(env, N, lanes, warps):
     b.close()
 
 
-def test_fields_beyond_the_fixed_point_range(env):
+@pytest.mark.parametrize("precision,lanes", [(0, 1), (1, 1), (1, 8)])
+def test_fields_beyond_the_fixed_point_range(env, precision, lanes):
     """A field too strong for the fixed-point pivots takes its group's slices through the FP64 sweep:
-    both kinds in one batch, and before and after the pulse, against the oracle."""
+    both kinds in one batch, and before and after the pulse, against the oracle (MIXED: its pivots)."""
     tdse, oracle = env
     N, dx, dt, a, nt = 512, 0.2, 0.05, 1.19, 96
     rows = [np.full(nt + 1, 0.02) for _ in range(40)]
@@ -920,17 +924,18 @@ def test_fields_beyond_the_fixed_point_range(env):
         rows[i][40:50] = 6.0
     offs = np.arange(41) * (nt + 1)
     Et = _device_rows(rows, offs, torch.device("cuda", 0))
-    b = tdse.Batch([N] * 40, dx, a, nt, dt, absorber=(20.0, 0.125), lanes_per_instance=1)
+    b = tdse.Batch([N] * 40, dx, a, nt, dt, absorber=(20.0, 0.125), lanes_per_instance=lanes, precision=precision)
     b.ground_state(**GS_KW)
     d, acc = torch.zeros_like(Et), torch.zeros_like(Et)
     b.propagate(Et, d, acc)
     assert b.check() == -1
     psi0, _, _ = oracle.ground_state(N, dx, a, **GS_KW)
     m = oracle.mask(N, dx, 20.0, 0.125)
+    bound = MIXED_SERIES if precision else RTOL_SERIES
     for i in (0, 1, 35, 39):
         _, d_o, a_o = oracle.propagate(psi0, rows[i], dx, dt, a, mask_values=m)
         sl = slice(offs[i], offs[i + 1])
-        assert _rel(d[sl].cpu().numpy(), d_o) < RTOL_SERIES and _rel(acc[sl].cpu().numpy(), a_o) < RTOL_SERIES, i
+        assert _rel(d[sl].cpu().numpy(), d_o) < bound and _rel(acc[sl].cpu().numpy(), a_o) < bound, i
     b.close()
 
 
