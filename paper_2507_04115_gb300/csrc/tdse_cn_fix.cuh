@@ -44,6 +44,96 @@ __device__ __forceinline__ FixSlot load_slot(const int4* __restrict__ p)
 // Is the group's shape one that fix_slice takes?  (m >= 4: a pass reads its own rows three ahead.)
 __device__ __forceinline__ bool fix_shape(const GroupDesc& G, const ClassDesc& C) { return C.fix.ok && G.m >= 4; }
 
+__device__ __forceinline__ ObsSums fix_lane_sum(ObsSums o, int I)
+{
+    for (int off = I; off < kLanes; off <<= 1) {
+        o.n += __shfl_xor_sync(0xffffffffu, o.n, off);
+        o.x += __shfl_xor_sync(0xffffffffu, o.x, off);
+        o.v += __shfl_xor_sync(0xffffffffu, o.v, off);
+    }
+    return o;
+}
+
+// Range of the slice's fields, norm and scale of the state: false when an instance is outside the
+// fixed-point range (the same answer on every warp).
+__device__ __forceinline__ bool fix_range(const GroupDesc& G, const FixClass& F, const double2* __restrict__ ps,
+                                          const double* __restrict__ E, int64_t row, int64_t nt, int64_t n0, int64_t n1,
+                                          int64_t sample_base, int s_own, int e_own, double* red, int& sigma)
+{
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, P = blockDim.x >> 5;
+    const int I = G.I, i = lane & (I - 1);
+    const bool live = nt > n0;
+    bool ok = true;
+    if (live)
+        for (int64_t n = n0; n <= min(n1, nt); ++n) ok = ok && fabs(E[row + n - sample_base]) <= F.E_lim;
+    float sq = 0.0f;
+    if (live)
+        for (int j = s_own; j < e_own; ++j) {
+            const double2 p = ld_cg(ps + (int64_t)j * I + i);
+            const float a = d2f(p.x), b = d2f(p.y);
+            sq = fmaf(a, a, fmaf(b, b, sq));
+        }
+    for (int off = I; off < kLanes; off <<= 1) sq += __shfl_xor_sync(0xffffffffu, sq, off);
+    float* redf = reinterpret_cast<float*>(red);
+    redf[w * kLanes + lane] = sq;
+    __syncthreads();
+    float tot = 0.0f;
+    for (int k = 0; k < P; ++k) tot += redf[k * kLanes + lane];
+    __syncthreads();
+    ok = ok && (!live || (tot > 1e-30f && tot < 1e30f));
+    // ||psi||^2 = f 2^e, f in [1, 2): 2^sigma puts the norm in [2^(top-1), 2^top)
+    const int e2 = live ? (int)((__float_as_uint(tot) >> 23) & 0xffu) - 127 : 0;
+    sigma = F.top - ((e2 + 2) >> 1);
+    return __all_sync(0xffffffffu, ok);
+}
+
+// Observables (and checkpoint 0) of the initial state.
+template <bool kCkpt>
+__device__ __forceinline__ void fix_initial(const GroupDesc& G, const ClassDesc& C, const double* __restrict__ tab,
+                                            const double2* __restrict__ ps, int64_t nt, int64_t row, int s_own, int e_own,
+                                            const double* __restrict__ E, double* __restrict__ d_out,
+                                            double* __restrict__ a_out, int64_t sample_base, double* red, double2* __restrict__ ck)
+{
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, P = blockDim.x >> 5;
+    const int I = G.I, i = lane & (I - 1);
+    const double dx = C.dx;
+    const double2* __restrict__ tab_xv2 = reinterpret_cast<const double2*>(tab + tab_xv(C));
+    ObsSums o{0.0, 0.0, 0.0};
+    for (int j = s_own; j < e_own; ++j) {
+        const double2 p = ld_cg(ps + (int64_t)j * I + i);
+        if constexpr (kCkpt) ck[(int64_t)j * I + i] = p;
+        const double rho = fma(p.x, p.x, p.y * p.y);
+        const double2 xv = __ldg(tab_xv2 + j);
+        o.n += rho;
+        o.x = fma(xv.x, rho, o.x);
+        o.v = fma(xv.y, rho, o.v);
+    }
+    const ObsSums t = reduce_obs(fix_lane_sum(o, I), red, P);
+    if (w == 0 && lane < I && nt >= 0) {
+        const double E0 = E[row - sample_base];
+        d_out[row - sample_base] = t.x * dx;
+        a_out[row - sample_base] = fma(E0, t.n, t.v) * dx;
+    }
+    __syncthreads();
+}
+
+// rho = |psi|^2 2^-60 in integers and its sums: over the points, times x in half grid steps (wj = 2 j - N + 1),
+// times dV (ob.x, ob.y: its digits); the last two as high and low parts.
+__device__ __forceinline__ void fix_observe(int64_t xr, int64_t xi, int wj, const int4& ob, int64_t& sn, int64_t& sxh,
+                                            int64_t& sxl, int64_t& svh, int64_t& svm)
+{
+    const Digits a = digits(xr), b = digits(xi);
+    const uint64_t ll = (uint64_t)mad(a.l, a.l, mad(b.l, b.l, 0)) >> 33;
+    const int64_t rho = combine<4, 27>(mad(a.h, a.h, mad(b.h, b.h, 0)),
+                                       mad(a.h, a.l, mad(b.h, b.l, (int64_t)ll + (int64_t(1) << 26))));
+    const Digits rd = digits(rho);
+    sn += rho;
+    sxh = mad(rd.h, wj, sxh);
+    sxl = mad(rd.l, wj, sxl);
+    svh = mad(rd.h, ob.y, svh) + (mad(rd.l, ob.y, int64_t(1) << 31) >> 32);
+    svm = mad(rd.h, ob.x, svm);
+}
+
 // Returns false, having changed nothing, when an instance's field or norm is outside the fixed-point
 // range of this slice (or not finite): the caller then takes the FP64 sweep.
 template <bool kCkpt>
@@ -67,58 +157,9 @@ __device__ __forceinline__ bool fix_slice(const GroupDesc& G, const ClassDesc& C
     const int4* __restrict__ tO = reinterpret_cast<const int4*>(tab + tab_fob(C));
 
     auto field = [&](int64_t n) { return n <= nt ? E[row + n - sample_base] : 0.0; };   // live lanes, n >= n0
-    // range of the fields of this slice, norm and scale of the state
-    bool ok = true;
-    if (live)
-        for (int64_t n = n0; n <= min(n1, nt); ++n) ok = ok && fabs(field(n)) <= F.E_lim;
-    float sq = 0.0f;
-    if (live)
-        for (int j = s_own; j < e_own; ++j) {
-            const double2 p = ld_cg(ps + (int64_t)j * I + i);
-            const float a = d2f(p.x), b = d2f(p.y);
-            sq = fmaf(a, a, fmaf(b, b, sq));
-        }
-    for (int off = I; off < kLanes; off <<= 1) sq += __shfl_xor_sync(0xffffffffu, sq, off);
-    float* redf = reinterpret_cast<float*>(red);
-    redf[w * kLanes + lane] = sq;
-    __syncthreads();
-    float tot = 0.0f;
-    for (int k = 0; k < P; ++k) tot += redf[k * kLanes + lane];
-    __syncthreads();
-    ok = ok && (!live || (tot > 1e-30f && tot < 1e30f));
-    if (!__all_sync(0xffffffffu, ok)) return false;
-    // ||psi||^2 = f 2^e, f in [1, 2): 2^sigma puts the norm in [2^(top-1), 2^top)
-    const int e2 = live ? (int)((__float_as_uint(tot) >> 23) & 0xffu) - 127 : 0;
-    const int sigma = F.top - ((e2 + 2) >> 1);
-
-    auto lane_sum = [&](ObsSums o) {
-        for (int off = I; off < kLanes; off <<= 1) {
-            o.n += __shfl_xor_sync(0xffffffffu, o.n, off);
-            o.x += __shfl_xor_sync(0xffffffffu, o.x, off);
-            o.v += __shfl_xor_sync(0xffffffffu, o.v, off);
-        }
-        return o;
-    };
-    if (initial) {   // observables (and checkpoint 0) of the initial state
-        const double2* __restrict__ tab_xv2 = reinterpret_cast<const double2*>(tab + tab_xv(C));
-        ObsSums o{0.0, 0.0, 0.0};
-        for (int j = s_own; j < e_own; ++j) {
-            const double2 p = ld_cg(ps + (int64_t)j * I + i);
-            if constexpr (kCkpt) ck[(int64_t)j * I + i] = p;
-            const double rho = fma(p.x, p.x, p.y * p.y);
-            const double2 xv = __ldg(tab_xv2 + j);
-            o.n += rho;
-            o.x = fma(xv.x, rho, o.x);
-            o.v = fma(xv.y, rho, o.v);
-        }
-        const ObsSums t = reduce_obs(lane_sum(o), red, P);
-        if (w == 0 && q == 0 && nt >= 0) {
-            const double E0 = E[row - sample_base];
-            d_out[row - sample_base] = t.x * dx;
-            a_out[row - sample_base] = fma(E0, t.n, t.v) * dx;
-        }
-        __syncthreads();
-    }
+    int sigma;
+    if (!fix_range(G, F, ps, E, row, nt, n0, n1, sample_base, s_own, e_own, red, sigma)) return false;
+    if (initial) fix_initial<kCkpt>(G, C, tab, ps, nt, row, s_own, e_own, E, d_out, a_out, sample_base, red, ck);
 
     // scales of the observable sums: rho_int = |psi|^2 2^(2 sigma - 60)
     const double unit = __hiloint2double((1023 + 60 - 2 * sigma) << 20, 0);   // |sigma| <= 112
@@ -280,20 +321,7 @@ __device__ __forceinline__ bool fix_slice(const GroupDesc& G, const ClassDesc& C
                 row_psi(j, nDr, nDi, xr, xi);
                 const bool in = (unsigned)j < (unsigned)N;
                 if (!in) xr = xi = 0;
-                // observables: rho 2^60 units, x in half grid steps
-                {
-                    const Digits a = digits(xr), b = digits(xi);
-                    const uint64_t ll = (uint64_t)mad(a.l, a.l, mad(b.l, b.l, 0)) >> 33;
-                    const int64_t rho = combine<4, 27>(mad(a.h, a.h, mad(b.h, b.h, 0)),
-                                                       mad(a.h, a.l, mad(b.h, b.l, (int64_t)ll + (int64_t(1) << 26))));
-                    const Digits rd = digits(rho);
-                    const int wj = 2 * j - N + 1;
-                    sn += rho;
-                    sxh = mad(rd.h, wj, sxh);
-                    sxl = mad(rd.l, wj, sxl);
-                    svh = mad(rd.h, ob.y, svh) + (mad(rd.l, ob.y, 0) >> 32);
-                    svm = mad(rd.h, ob.x, svm);
-                }
+                fix_observe(xr, xi, 2 * j - N + 1, ob, sn, sxh, sxl, svh, svm);
                 if (any_put && in) {
                     const double2 v = make_double2(__longlong_as_double((long long)fix_to_double(xr, sigma)),
                                                    __longlong_as_double((long long)fix_to_double(xi, sigma)));
@@ -316,7 +344,235 @@ __device__ __forceinline__ bool fix_slice(const GroupDesc& G, const ClassDesc& C
             o.x = fma((double)sxh, two32, (double)sxl) * (0.5 * dx * unit);
             o.v = fma((double)svh, two32, (double)svm) * (two32 * F.v_scale * unit);
         }
-        const ObsSums t = reduce_obs(lane_sum(o), red, P);   // its barrier orders this pass's writes
+        const ObsSums t = reduce_obs(fix_lane_sum(o, I), red, P);   // its barrier orders this pass's writes
+        if (w == 0 && q == 0 && active) {
+            const int64_t kk = row + n + 1 - sample_base;
+            d_out[kk] = t.x * dx;
+            a_out[kk] = fma(En1, t.n, t.v) * dx;
+            if (!(t.n * dx <= 1.0 + 1e-6)) status[slot] = 1;
+        }
+    }
+    return true;
+}
+
+// The same step for short segments (lane-split groups, m <= 4 K), where fix_slice's lead-in of 2K rows
+// would cost several times the m own rows.  D and Y are affine in the value that enters a segment,
+//     D_r = D^0_r + H_r D_in,  Y_r = Y^0_r + (prod_{k>=r} gamma_k) Y_in,  H_r = prod_{k<=r} gamma_k,
+// so each segment runs from zero, publishes its outgoing D^0, Y^0 and its product H in shared memory, and
+// composes what enters from the T = ceil(K / m) segments before (after) it; farther ones are below beta^K.
+// Only gamma, whose recurrence is not linear, has a lead-in, and as its error falls by gamma^2 a row, K/2
+// rows of it.  Then the first min(m, K) rows of D are run again from D_in, and all of Y from Y_in.
+// psi (integers, converted once per slice), gamma and D of the own rows stay in the CTA's scratch, 1.5 KB a
+// row and warp, which small batches find in L1.
+// Measured, one atom (N = 2000, K = 36, 512 steps): 18.6 ms with fix_slice (4 warps), 8.3 here (6 warps); the uneven
+// scan 19.5 ms and 15.0.
+struct FixEdge {   // per column of the CTA
+    int64_t dr, di;
+    Digits hr, hi;
+    int64_t yr, yi;
+};
+
+static_assert(sizeof(FixEdge) == kEdgeBytes, "shared memory of the launch");
+
+__device__ __forceinline__ bool fix_short(const GroupDesc& G) { return G.I != kLanes && G.K > 0 && G.m <= 4 * G.K; }
+
+template <bool kCkpt>
+__device__ __forceinline__ bool fix_short_slice(const GroupDesc& G, const ClassDesc& C, const double* __restrict__ tab,
+                                                double2* __restrict__ ps, int64_t nt, int64_t row, int64_t slot, int64_t n0,
+                                                int64_t n1, bool initial, const double* __restrict__ E,
+                                                double* __restrict__ d_out, double* __restrict__ a_out, int64_t sample_base,
+                                                int4* __restrict__ buf, double* red, FixEdge* edge, int* status,
+                                                double2* __restrict__ ck, int kc, int jm_lo, int jm_hi)
+{
+    const FixClass& F = C.fix;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, P = blockDim.x >> 5;
+    const int I = G.I, i = lane & (I - 1), q = lane / I;
+    const int N = G.N, K = G.K, m = G.m, Kg = (K + 1) / 2, Kr = min(m, K), T = (K + m - 1) / m;
+    const bool on = w < G.P;
+    const int sg = w * (kLanes / I) + q, n_seg = G.P * (kLanes / I);   // this lane's segment
+    const int s = sg * m, col = w * kLanes + lane;
+    const int s_own = on ? min(N, s) : N, e_own = on ? min(N, s + m) : N;
+    const bool live = nt > n0;
+    const double dx = C.dx;
+    const int4* __restrict__ tT = reinterpret_cast<const int4*>(tab + tab_fxp(C));
+    const int4* __restrict__ tO = reinterpret_cast<const int4*>(tab + tab_fob(C));
+    auto field = [&](int64_t n) { return n <= nt ? E[row + n - sample_base] : 0.0; };
+    int sigma;
+    if (!fix_range(G, F, ps, E, row, nt, n0, n1, sample_base, s_own, e_own, red, sigma)) return false;
+    if (initial) fix_initial<kCkpt>(G, C, tab, ps, nt, row, s_own, e_own, E, d_out, a_out, sample_base, red, ck);
+
+    const double unit = __hiloint2double((1023 + 60 - 2 * sigma) << 20, 0);   // |sigma| <= 112
+    const int64_t inv_b = F.inv_b;
+    const int32_t ci = F.ci;
+    const Digits cf = F.cf;
+    int4* __restrict__ own = buf + (int64_t)w * m * (3 * kLanes) + lane;   // row r: gamma, psi, D at own + r * 96 + (0, 32, 64)
+    auto put64 = [](int4* p, int64_t a, int64_t b) {
+        *p = make_int4((int)(uint32_t)(uint64_t)a, (int)(uint32_t)((uint64_t)a >> 32), (int)(uint32_t)(uint64_t)b,
+                       (int)(uint32_t)((uint64_t)b >> 32));
+    };
+    auto lo64 = [](const int4& v) { return (int64_t)(((uint64_t)(uint32_t)v.y << 32) | (uint32_t)v.x); };
+    auto hi64 = [](const int4& v) { return (int64_t)(((uint64_t)(uint32_t)v.w << 32) | (uint32_t)v.z); };
+    auto gam = [](const int4& v, Digits& r, Digits& m_) {
+        r = Digits{v.x, v.y};
+        m_ = Digits{v.z, v.w};
+    };
+    if (on)
+        for (int r = 0; r < m; ++r) {
+            const int j = s + r;
+            const double2 p = live && j < N ? ld_cg(ps + (int64_t)j * I + i) : make_double2(0.0, 0.0);
+            put64(own + r * (3 * kLanes) + kLanes, double_to_fix((uint64_t)__double_as_longlong(p.x), sigma),
+                  double_to_fix((uint64_t)__double_as_longlong(p.y), sigma));
+        }
+    auto table = [&](int j) { return __ldg(tT + min(max(j, 0), N - 1)); };
+
+    for (int64_t n = n0; n < n1; ++n) {
+        const bool active = n < nt, last = n + 1 == n1;
+        const double En1 = active ? field(n + 1) : 0.0;
+        const bool put = active && (last || n + 1 == nt);
+        bool put_ck = false;
+        if constexpr (kCkpt) put_ck = (n + 1) % kc == 0 && n + 1 < G.nt_max;
+        const bool any_put = __any_sync(0xffffffffu, put) || put_ck;
+        const Digits Eb = digits(live && n < nt ? __double2ll_rn(0.5 * (field(n) + field(n + 1)) * F.e_scale) : 0);
+
+        // gamma (lead-in and own rows) and D from zero, ascending
+        if (on) {
+            int64_t gr = 0, gi = 0, dr = 0, di = 0;
+            int4 tn = table(s - Kg);
+            for (int r = -Kg; r < 0; ++r) {
+                const int4 t = tn;
+                tn = table(s + r + 1);
+                gamma_row(inv_b, diag_row(FixPoint{t.x, t.y, t.z, t.w}, Eb), gr, gi);
+                if (s + r < 0) gr = gi = 0;   // (a segment's lead-in never lies beyond the far wall unless it does itself)
+            }
+            Digits hr{0, 0}, hi{0, 0};
+            int4 pn = own[kLanes];
+            int4* o = own;
+            for (int r = 0; r < m; ++r) {
+                const int4 t = tn, p = pn;
+                tn = table(s + r + 1);
+                if (r + 1 < m) pn = o[4 * kLanes];
+                gamma_row(inv_b, diag_row(FixPoint{t.x, t.y, t.z, t.w}, Eb), gr, gi);
+                if (s + r >= N) gr = gi = 0;
+                const Digits a = digits(gr << 6), b = digits(gi << 6);
+                mul_minus_i(a, b, digits(lo64(p) - di), digits(hi64(p) + dr), dr, di);
+                o[0] = make_int4(a.h, a.l, b.h, b.l);
+                if (r >= Kr) put64(o + 2 * kLanes, dr, di);
+                if (T > 1) {   // H: product of the segment's gamma
+                    if (r == 0) {
+                        hr = a;
+                        hi = b;
+                    } else {
+                        const int64_t x = mul2_fix(a, hr, negative(b), hi), y = mul2_fix(a, hi, b, hr);
+                        hr = digits(x);
+                        hi = digits(y);
+                    }
+                }
+                o += 3 * kLanes;
+            }
+            edge[col].dr = dr;
+            edge[col].di = di;
+            edge[col].hr = hr;
+            edge[col].hi = hi;
+        }
+        __syncthreads();
+        // D entering the segment, D of its first Kr rows again, Y of those rows from zero
+        if (on) {
+            int64_t dr = 0, di = 0;
+            for (int k = min(T, sg); k >= 1; --k) {
+                const FixEdge& e = edge[col - k * I];
+                const Digits a = digits(dr), b = digits(di);
+                const int64_t x = mul2_fix(e.hr, a, negative(e.hi), b, e.dr), y = mul2_fix(e.hr, b, e.hi, a, e.di);
+                dr = x;
+                di = y;
+            }
+            int4* o = own;
+            int4 gn = o[0], pn = o[kLanes];
+            for (int r = 0; r < Kr; ++r) {
+                const int4 g = gn, p = pn;
+                if (r + 1 < Kr) {
+                    gn = o[3 * kLanes];
+                    pn = o[4 * kLanes];
+                }
+                Digits a, b;
+                gam(g, a, b);
+                mul_minus_i(a, b, digits(lo64(p) - di), digits(hi64(p) + dr), dr, di);
+                put64(o + 2 * kLanes, dr, di);
+                o += 3 * kLanes;
+            }
+            int64_t yr = 0, yi = 0;
+            o -= 3 * kLanes;
+            gn = o[0];
+            pn = o[2 * kLanes];
+            for (int r = Kr - 1; r >= 0; --r) {
+                const int4 g = gn, d = pn;
+                if (r > 0) {
+                    gn = o[-3 * kLanes];
+                    pn = o[-kLanes];
+                }
+                Digits a, b;
+                gam(g, a, b);
+                const Digits u = digits(yr), v = digits(yi);
+                yr = mul2_fix(a, u, negative(b), v, lo64(d));
+                yi = mul2_fix(a, v, b, u, hi64(d));
+                o -= 3 * kLanes;
+            }
+            edge[col].yr = yr;
+            edge[col].yi = yi;
+        }
+        __syncthreads();
+        // Y entering the segment, then the whole segment, descending: psi^{n+1} and the observables
+        ObsSums ob_sum{0.0, 0.0, 0.0};
+        if (on) {
+            int64_t yr = 0, yi = 0;
+            for (int k = min(T, n_seg - 1 - sg); k >= 1; --k) {
+                const FixEdge& e = edge[col + k * I];
+                const Digits a = digits(yr), b = digits(yi);
+                const int64_t x = mul2_fix(e.hr, a, negative(e.hi), b, e.yr), y = mul2_fix(e.hr, b, e.hi, a, e.yi);
+                yr = x;
+                yi = y;
+            }
+            int64_t sn = 0, sxh = 0, sxl = 0, svh = 0, svm = 0;
+            int4* o = own + (int64_t)(m - 1) * (3 * kLanes);
+            int4 gn = o[0], pn = o[kLanes], dn = o[2 * kLanes];
+            int4 obn = __ldg(tO + min(s + m - 1, N - 1));
+            for (int r = m - 1; r >= 0; --r) {
+                const int j = s + r;
+                const int4 g = gn, p = pn, d = dn, ob = obn;
+                if (r > 0) {
+                    gn = o[-3 * kLanes];
+                    pn = o[-2 * kLanes];
+                    dn = o[-kLanes];
+                    obn = __ldg(tO + min(j - 1, N - 1));
+                }
+                Digits a, b;
+                gam(g, a, b);
+                const Digits u = digits(yr), v = digits(yi);
+                yr = mul2_fix(a, u, negative(b), v, lo64(d));
+                yi = mul2_fix(a, v, b, u, hi64(d));
+                int64_t xr = update_fix(ci, cf, digits(yr), lo64(p)), xi = update_fix(ci, cf, digits(yi), hi64(p));
+                if (j < jm_lo || j > jm_hi) {
+                    const Digits mm{ob.w, ob.z};
+                    xr = mul_fix<3>(mm, digits(xr));
+                    xi = mul_fix<3>(mm, digits(xi));
+                }
+                if (j >= N) xr = xi = 0;
+                put64(o + kLanes, xr, xi);
+                fix_observe(xr, xi, 2 * j - N + 1, ob, sn, sxh, sxl, svh, svm);
+                if (any_put && j < N) {
+                    const double2 z = make_double2(__longlong_as_double((long long)fix_to_double(xr, sigma)),
+                                                   __longlong_as_double((long long)fix_to_double(xi, sigma)));
+                    if (put) ps[(int64_t)j * I + i] = z;
+                    if constexpr (kCkpt)
+                        if (put_ck) ck[((n + 1) / kc) * ((int64_t)N * I) + (int64_t)j * I + i] = z;
+                }
+                o -= 3 * kLanes;
+            }
+            const double two32 = 4294967296.0;
+            ob_sum.n = (double)sn * unit;
+            ob_sum.x = fma((double)sxh, two32, (double)sxl) * (0.5 * dx * unit);
+            ob_sum.v = fma((double)svh, two32, (double)svm) * (two32 * F.v_scale * unit);
+        }
+        const ObsSums t = reduce_obs(fix_lane_sum(ob_sum, I), red, P);
         if (w == 0 && q == 0 && active) {
             const int64_t kk = row + n + 1 - sample_base;
             d_out[kk] = t.x * dx;

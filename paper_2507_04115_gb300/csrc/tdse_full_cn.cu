@@ -313,7 +313,13 @@ k_propagate_full_cn(const GroupDesc* __restrict__ groups, int64_t n_groups, cons
 
         bool done = false;
         if constexpr (!kMixed)
-            if (fix_shape(G, C))
+            if (C.fix.ok && fix_short(G))
+                done = fix_short_slice<kCkpt>(G, C, tab, ps, nt, row, slot, n0, n1, kslice == 0 && step_begin == 0, E, d_out,
+                                              a_out, sample_base,
+                                              reinterpret_cast<int4*>(scratch_raw) + (int64_t)blockIdx.x * P * rows * (2 * kLanes),
+                                              red, reinterpret_cast<FixEdge*>(red + P * 3 * kLanes), status,
+                                              kCkpt ? ckpt + ckpt_off[g] : nullptr, kc, jm_lo, jm_hi);
+            else if (fix_shape(G, C))
                 done = fix_slice<kCkpt>(G, C, tab, ps, nt, row, slot, n0, n1, kslice == 0 && step_begin == 0, E, d_out, a_out,
                                         sample_base, reinterpret_cast<int4*>(scratch_raw) + (int64_t)blockIdx.x * P * rows * (2 * kLanes),
                                         red, status, kCkpt ? ckpt + ckpt_off[g] : nullptr, kc, jm_lo, jm_hi);

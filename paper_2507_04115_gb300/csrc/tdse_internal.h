@@ -138,14 +138,18 @@ inline double group_step_cost(int N, int K, int L, int warps)
 // units, W the warps that share the SM (at least 4, one per sub-partition): its latency, hidden by the
 // other warps as far as they are, and everyone's instructions.  Measured, volume batch (K = 28, 160
 // steps): 120 ms at 8 warps, 104 at 12, 100 at 16, 113 with two CTAs of 8; one atom (K = 36, L = 32, 512
-// steps): 23.7 ms at 2 warps, 18.8 at 4, 20.9 at 8.
+// steps, short segments): 14.9 ms at 2 warps, 9.2 at 4, 8.9 at 6, 9.5 at 8, 9.8 at 16.
 // `lead`: whole rows' worth of a halo row, 1.3 there; 0.6 for NUMEROV_SPLIT (tdse_numerov_fix.cuh), whose
 // lead-ins run one sweep each.
 constexpr double kLeadFullCn = 1.3, kLeadNumerov = 0.6;
 inline double fix_step_cost(int N, int K, int L, int P, int W, double lead)
 {
     const int m = group_segment_length(N, P, L);
-    return 0.17 * (6.0 + std::max(W, 4)) * (m + lead * (P * L > 1 ? K : 0));
+    double rows = m + lead * (P * L > 1 ? K : 0);
+    // short segments of lane-split FULL_CN groups (fix_short_slice): a light lead-in, part of the rows run
+    // again, and the composition over ceil(K / m) segments
+    if (lead == kLeadFullCn && L > 1 && K > 0 && m <= 4 * K) rows = m + 0.15 * K + 0.3 * std::min(m, K) + (K + m - 1) / m;
+    return 0.17 * (6.0 + std::max(W, 4)) * rows;
 }
 // Warps carrying segments there when `per_sm` CTAs share an SM: the cheapest of those that group_warps
 // allows, segments of at least 4 points (a pass reads its own rows three ahead).

@@ -32,9 +32,13 @@ inline int full_cn_ring_slots(int P, int per_sm)
     return r < kMinRing ? kMinRing : (r > kMaxRing ? kMaxRing : (int)r);
 }
 
+// Values that leave a segment of the fixed-point sweep's short-segment form, per lane (FixEdge).
+constexpr int kEdgeBytes = 48;
+
 __host__ __device__ inline size_t full_cn_smem_bytes(int mixed, int P, int ring)
 {
     size_t b = (size_t)P * 3 * 32 * sizeof(double);
+    if (!mixed) b += (size_t)P * 32 * kEdgeBytes;
     if (mixed) b += (size_t)P * ring * (sizeof(uint64_t) + kSlotBytes);
     return b;
 }
