@@ -22,7 +22,7 @@
 //   k_field_interp  16 multiply-adds per output
 // Work per row: O(M^2 / 2 + G log G + 16 n_fine) FP64 instructions instead of O(3 M^2 + 3 M n_fine) for the
 // direct sums with turning twiddles.  Measured, 256 rows of 2400 samples to 55160: 217 ms by the direct
-// sums, 2.9 ms here, of which the FP64 pipe needs 1.2 (coefficients) and 0.4 (interpolation).
+// sums, 2.9 ms here: coefficients 1.8, tables 0.4, interpolation 0.4, grid 0.15.
 #include "tdse_device.cuh"
 #include "tdse_internal.h"
 
@@ -35,15 +35,17 @@ constexpr int kInterpRows = 8;      // rows per thread of the interpolation
 constexpr int kGridThreads = 512;
 constexpr double kPi = 3.14159265358979323846;
 
-// b sqrt(1 - y^2) -> I0 by its power series (all terms positive)
-__device__ double bessel_i0(double x)
+// I0(x), |x| <= 16 pi, by its power series (all terms positive), r[k] = 1 / k^2: a division per term would be
+// most of the work
+constexpr int kI0Terms = 100;
+__device__ double bessel_i0(double x, const double* r)
 {
     const double h = 0.25 * x * x;
     double t = 1.0, s = 1.0;
-    for (int k = 1; k < 120; ++k) {
-        t *= h / ((double)k * k);
+    for (int k = 1; k < kI0Terms; ++k) {
+        t *= h * r[k];
         s += t;
-        if (t < 1e-18 * s) break;
+        if (__double2hiint(t) + (60 << 20) < __double2hiint(s)) break;   // below 2^-60 of the sum
     }
     return s;
 }
@@ -51,6 +53,9 @@ __device__ double bessel_i0(double x)
 __global__ void k_field_tables(int M, int G, double b, double dt_f, double T, int64_t n_fine, double2* __restrict__ tw_m,
                                double2* __restrict__ tw_g, int* __restrict__ node, double* __restrict__ wgt)
 {
+    __shared__ double inv_k2[kI0Terms];
+    for (int k = threadIdx.x; k < kI0Terms; k += blockDim.x) inv_k2[k] = k > 0 ? 1.0 / ((double)k * k) : 0.0;
+    __syncthreads();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < M) {   // e^{2 pi i j / M}
         double s, c;
@@ -72,7 +77,7 @@ __global__ void k_field_tables(int M, int G, double b, double dt_f, double T, in
         const double z = (xh - l) + ql * G;            // offset from node l, in [0, 1] to rounding
         const double y = (z + (kWin / 2 - 1) - j) * (2.0 / kWin);
         const double r = 1.0 - y * y;
-        wgt[j * n_fine + n] = r > 0.0 ? bessel_i0(b * sqrt(r)) : 0.0;   // phi up to the factor in k_field_grid
+        wgt[j * n_fine + n] = r > 0.0 ? bessel_i0(b * sqrt(r), inv_k2) : 0.0;   // phi up to the factor in k_field_grid
         if (j == 0) node[n] = ((int)l - (kWin / 2 - 1) + G) & (G - 1);
     }
 }
