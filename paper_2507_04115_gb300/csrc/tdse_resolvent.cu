@@ -73,19 +73,28 @@ __global__ void k_ed_pivots(const ClassDesc* __restrict__ cls, int n_cls, const 
     const double zr = k < nE ? E_grid[k] : 0.0, zi = -eps;
     double2* W = pivW + piv_off[c];
     double2* Cp = pivC + piv_off[c];
+    if (scheme == 0) {
+        // in units of the off-diagonal a: v_j = c'_j = 1 / (b_j / a - v_{j-1}), a chain of 8 dependent
+        // instructions a row (they set the time: 128 energies are 4 warps)
+        const double inv_a = 2.0 * C.dx * C.dx, bi = zi * inv_a;
+        double2 v = make_double2(0.0, 0.0);
+        double Vn = V[0];
+        for (int j = 0; j < N; ++j) {
+            const double br = (zr - (inv_dx2 + Vn)) * inv_a;
+            if (j + 1 < N) Vn = V[j + 1];
+            v = cinv(make_double2(br - v.x, bi - v.y));
+            Cp[(int64_t)j * nE_pad + k] = v;
+        }
+        return;
+    }
     double2 cprev = make_double2(0.0, 0.0);
     for (int j = 0; j < N; ++j) {
         const EdRow r = ed_row(scheme, zr, zi, inv_dx2, V, j, N);
         const double2 ac = cmul(r.a, cprev);
         const double2 w = make_double2(r.b.x - ac.x, r.b.y - ac.y);
         const double2 iw = cinv(w);
-        if (scheme == 0) {   // a / w_j, which is c'_j but for the last row (see k_ed_solve)
-            const double a = 0.5 * inv_dx2;
-            cprev = make_double2(a * iw.x, a * iw.y);
-        } else {
-            cprev = cmul(r.c, iw);
-            W[(int64_t)j * nE_pad + k] = iw;
-        }
+        cprev = cmul(r.c, iw);
+        W[(int64_t)j * nE_pad + k] = iw;
         Cp[(int64_t)j * nE_pad + k] = cprev;
     }
 }
