@@ -422,12 +422,13 @@ cudaError_t launch_adjoint_full_cn(const GroupDesc* d_groups, int64_t n_groups, 
                                    const void* d_psi0, void* d_lam, void* d_ckpt, const int64_t* d_ckpt_off,
                                    void* d_work, void* d_tape, void* d_scratch, int rows, int n_max, int kc,
                                    const double* E, const double* gd, const double* ga, double* gE, int mask_on,
-                                   int* d_busy, int* d_progress, cudaStream_t st, int have_ckpt, void* d_gtape)
+                                   int* d_busy, int* d_progress, cudaStream_t st, int have_ckpt, void* d_gtape, int* d_left)
 {
     if (n_groups == 0 || ctas == 0) return cudaSuccess;
     cudaError_t e = cudaMemsetAsync(d_busy, 0, sizeof(int) * n_groups, st);
     if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(d_progress, 0, sizeof(int) * n_groups, st);
+    if (d_left) d_progress = d_left;   // 1: the group is done
+    else e = cudaMemsetAsync(d_progress, 0, sizeof(int) * n_groups, st);
     if (e != cudaSuccess) return e;
     const size_t smem = (size_t)P * 3 * kLanes * sizeof(double);
     k_adjoint_full_cn<<<(unsigned)ctas, P * kLanes, smem, st>>>(

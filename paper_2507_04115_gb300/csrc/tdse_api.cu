@@ -130,10 +130,12 @@ struct tdse_batch {
     size_t gtape_bytes = 0;
     bool use_gtape = true;             // tdse_set_adjoint_gamma_tape
     int adj_kc = 0, adj_ctas = 0;
-    // launch shape of the adjoint kernel (its sweeps are in double: the rules of that pipe)
+    // launch shape of the adjoint kernels (one CTA per SM: the fixed-point rules where a class has that form)
     std::vector<GroupDesc> adj_groups;
     GroupDesc* d_adj_groups = nullptr;
     int adj_warps = 8, adj_rows = 0, adj_grid = 0;
+    int64_t adj_fix_scratch = 0;   // per CTA; 0: no group with the fixed-point form
+    int* d_left = nullptr;         // groups that it leaves to the FP64 kernel
     // checkpoints recorded by tdse_propagate_checkpointed: steps [0, ckpt_next) are covered (-1: none)
     int64_t ckpt_next = -1;
     // energy-distribution buffers (allocated on first use, grown as needed)
@@ -176,6 +178,8 @@ void free_device(tdse_batch* b)
     cudaFree(b->d_ed_scratch);
     cudaFree(b->d_adj_groups);
     b->d_adj_groups = nullptr;
+    cudaFree(b->d_left);
+    b->d_left = nullptr;
     b->d_slot_group = b->d_slot_inst = nullptr;
     b->d_ed_scratch = nullptr;
     b->ed_scratch_elems = 0;
@@ -555,11 +559,19 @@ tdse_status build_plan(tdse_batch* b)
     b->ctas = grid(per_sm);
     int64_t sc = (int64_t)b->ctas * b->warps * b->rows * 2 * kLanes;
     if (b->precision == TDSE_FP64 && b->scheme == TDSE_FULL_CN) {
-        // the adjoint kernel's shape; it shares the scratch
+        // the adjoint kernels' shape; they share the scratch
         b->adj_groups = b->groups;
-        b->adj_rows = shape_groups(b, b->adj_groups, false, 1, &b->adj_warps);
+        b->adj_rows = shape_groups(b, b->adj_groups, fix, 1, &b->adj_warps);
         b->adj_grid = grid(b->ctas_per_sm_override > 0 ? std::min(b->ctas_per_sm_override, propagate_max_ctas_per_sm(0, b->adj_warps)) : 1);
         sc = std::max(sc, (int64_t)b->adj_grid * b->adj_warps * b->adj_rows * 2 * kLanes);
+        b->adj_fix_scratch = 0;
+        for (const GroupDesc& G : b->adj_groups)
+            if (on_fix_path(b, b->classes[G.cls]) && G.K > 0)
+                b->adj_fix_scratch = std::max(b->adj_fix_scratch, adjoint_fix_scratch(b->adj_warps, G.m));
+        sc = std::max(sc, (int64_t)b->adj_grid * b->adj_fix_scratch);
+        cudaFree(b->d_left);
+        b->d_left = nullptr;
+        TDSE_CUDA(dev_alloc(&b->d_left, b->adj_groups.size()), "cudaMalloc(sched)");
         cudaFree(b->d_adj_groups);
         b->d_adj_groups = nullptr;
         TDSE_CUDA(dev_alloc(&b->d_adj_groups, b->adj_groups.size()), "cudaMalloc(groups)");
@@ -644,6 +656,32 @@ void ensure_gamma_tape(tdse_batch* b, int kc)
         return;
     }
     b->gtape_bytes = need;
+}
+
+// The adjoint's kernels: the fixed-point one where a class has that form, then the FP64 one for what it leaves (all
+// groups when no class has it, or the interval is too long for its per-sample sums; only then is the gamma tape
+// worth its memory).
+tdse_status adjoint_launches(tdse_batch* b, const double* E, const double* gd, const double* ga, double* gE, int n_max, int kc,
+                             cudaStream_t st, int have_ckpt)
+{
+    const int64_t n = (int64_t)b->groups.size();
+    int* left = nullptr;
+    if (b->adj_fix_scratch > 0 && kc < n_max) {
+        left = b->d_left;
+        TDSE_CUDA(launch_adjoint_fix(b->d_adj_groups, n, b->adj_warps, b->adj_grid, b->d_cls, b->d_tab, b->d_slot_row, b->d_slot_nt,
+                                     b->d_psi, b->d_lam, b->d_ckpt, b->d_ckpt_off, b->d_work, b->d_tape, b->d_scratch,
+                                     b->adj_fix_scratch, n_max, kc, E, gd, ga, gE, b->mask_on, b->d_busy, b->d_progress, left, st,
+                                     have_ckpt),
+                  "adjoint launch");
+    } else if (b->use_gtape) {
+        ensure_gamma_tape(b, kc);
+    }
+    TDSE_CUDA(launch_adjoint_full_cn(b->d_adj_groups, n, b->adj_warps, b->adj_grid, b->d_cls, b->d_tab, b->d_slot_row, b->d_slot_nt,
+                                     b->d_psi, b->d_lam, b->d_ckpt, b->d_ckpt_off, b->d_work, b->d_tape, b->d_scratch, b->adj_rows,
+                                     n_max, kc, E, gd, ga, gE, b->mask_on, b->d_busy, b->d_progress, st, have_ckpt,
+                                     b->use_gtape && !left ? b->d_gtape : nullptr, left),
+              "adjoint launch");
+    return TDSE_OK;
 }
 
 }  // namespace
@@ -1073,14 +1111,7 @@ tdse_status tdse_adjoint(tdse_batch* b, const double* E_dev, const double* gd_de
     tdse_status s = ensure_adjoint_buffers(b, ckpt_every, st, &n_max);
     if (s != TDSE_OK) return s;
     b->ckpt_next = -1;   // the adjoint's own forward pass rewrites the checkpoints
-    if (b->use_gtape) ensure_gamma_tape(b, ckpt_every);
-    TDSE_CUDA(launch_adjoint_full_cn(b->d_adj_groups, (int64_t)b->groups.size(), b->adj_warps, b->adj_grid, b->d_cls, b->d_tab,
-                                     b->d_slot_row, b->d_slot_nt, b->d_psi, b->d_lam, b->d_ckpt, b->d_ckpt_off,
-                                     b->d_work, b->d_tape, b->d_scratch, b->adj_rows, n_max, ckpt_every, E_dev, gd_dev,
-                                     ga_dev, gE_dev, b->mask_on, b->d_busy, b->d_progress, st, 0,
-                                     b->use_gtape ? b->d_gtape : nullptr),
-              "adjoint launch");
-    return TDSE_OK;
+    return adjoint_launches(b, E_dev, gd_dev, ga_dev, gE_dev, n_max, ckpt_every, st, 0);
 }
 
 tdse_status tdse_propagate_checkpointed(tdse_batch* b, const double* E_dev, double* d_dev, double* a_dev,
@@ -1136,14 +1167,7 @@ tdse_status tdse_adjoint_checkpointed(tdse_batch* b, const double* E_dev, const 
     if (b->ckpt_next < nt_all || !b->d_ckpt)
         return fail(TDSE_ERR_STATE, "tdse_adjoint_checkpointed: no complete checkpointed forward propagation "
                                     "(tdse_propagate_checkpointed from step 0 through every instance's last step)");
-    if (b->use_gtape) ensure_gamma_tape(b, b->adj_kc);
-    TDSE_CUDA(launch_adjoint_full_cn(b->d_adj_groups, (int64_t)b->groups.size(), b->adj_warps, b->adj_grid, b->d_cls, b->d_tab,
-                                     b->d_slot_row, b->d_slot_nt, b->d_psi, b->d_lam, b->d_ckpt, b->d_ckpt_off,
-                                     b->d_work, b->d_tape, b->d_scratch, b->adj_rows, n_max, b->adj_kc, E_dev, gd_dev,
-                                     ga_dev, gE_dev, b->mask_on, b->d_busy, b->d_progress, st, 1,
-                                     b->use_gtape ? b->d_gtape : nullptr),
-              "adjoint launch");
-    return TDSE_OK;
+    return adjoint_launches(b, E_dev, gd_dev, ga_dev, gE_dev, n_max, b->adj_kc, st, 1);
 }
 
 

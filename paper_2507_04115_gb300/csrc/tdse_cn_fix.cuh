@@ -376,6 +376,151 @@ static_assert(sizeof(FixEdge) == kEdgeBytes, "shared memory of the launch");
 
 __device__ __forceinline__ bool fix_short(const GroupDesc& G) { return G.I != kLanes && G.K > 0 && G.m <= 4 * G.K; }
 
+// Geometry of a lane's segment in the short-segment form, and the own rows' scratch: row r holds gamma (digits),
+// the right-hand side and D (64-bit pairs) at own + r * 96 + (0, 32, 64).
+struct ShortGeom {
+    int N, K, m, I, s, sg, n_seg, col;
+    bool on;
+    int4* own;
+    FixEdge* edge;
+    const int4* tT;
+    int64_t inv_b;
+};
+__device__ __forceinline__ void put64(int4* p, int64_t a, int64_t b)
+{
+    *p = make_int4((int)(uint32_t)(uint64_t)a, (int)(uint32_t)((uint64_t)a >> 32), (int)(uint32_t)(uint64_t)b,
+                   (int)(uint32_t)((uint64_t)b >> 32));
+}
+__device__ __forceinline__ int64_t lo64(const int4& v) { return (int64_t)(((uint64_t)(uint32_t)v.y << 32) | (uint32_t)v.x); }
+__device__ __forceinline__ int64_t hi64(const int4& v) { return (int64_t)(((uint64_t)(uint32_t)v.w << 32) | (uint32_t)v.z); }
+__device__ __forceinline__ void gam(const int4& v, Digits& r, Digits& i)
+{
+    r = Digits{v.x, v.y};
+    i = Digits{v.z, v.w};
+}
+// (yr, yi) <- D + gamma Y at a row
+__device__ __forceinline__ void back_row(const int4& g, const int4& d, int64_t& yr, int64_t& yi)
+{
+    Digits a, b;
+    gam(g, a, b);
+    const Digits u = digits(yr), v = digits(yi);
+    yr = mul2_fix(a, u, negative(b), v, lo64(d));
+    yi = mul2_fix(a, v, b, u, hi64(d));
+}
+
+// The elimination of A y = rhs over the whole group, leaving gamma and D of every own row in the scratch and
+// the Y that enters this segment from the next ones in (yr, yi).  Two barriers inside; the caller's own
+// rows may be overwritten right after, the edges only after another barrier.
+__device__ __forceinline__ void short_solve(const ShortGeom& G, Digits Eb, int64_t& y_in_r, int64_t& y_in_i)
+{
+    const int N = G.N, K = G.K, m = G.m, I = G.I, s = G.s, sg = G.sg, n_seg = G.n_seg, col = G.col;
+    const int Kg = (K + 1) / 2, Kr = min(m, K), T = (K + m - 1) / m;
+    const bool on = G.on;
+    int4* const own = G.own;
+    FixEdge* const edge = G.edge;
+    const int64_t inv_b = G.inv_b;
+    auto table = [&](int j) { return __ldg(G.tT + min(max(j, 0), N - 1)); };
+    // gamma (lead-in and own rows) and D from zero, ascending
+    if (on) {
+        int64_t gr = 0, gi = 0, dr = 0, di = 0;
+        int4 tn = table(s - Kg);
+        for (int r = -Kg; r < 0; ++r) {
+            const int4 t = tn;
+            tn = table(s + r + 1);
+            gamma_row(inv_b, diag_row(FixPoint{t.x, t.y, t.z, t.w}, Eb), gr, gi);
+            if (s + r < 0) gr = gi = 0;   // (a segment's lead-in never lies beyond the far wall unless it does itself)
+        }
+        Digits hr{0, 0}, hi{0, 0};
+        int4 pn = own[kLanes];
+        int4* o = own;
+        for (int r = 0; r < m; ++r) {
+            const int4 t = tn, p = pn;
+            tn = table(s + r + 1);
+            if (r + 1 < m) pn = o[4 * kLanes];
+            gamma_row(inv_b, diag_row(FixPoint{t.x, t.y, t.z, t.w}, Eb), gr, gi);
+            if (s + r >= N) gr = gi = 0;
+            const Digits a = digits(gr << 6), b = digits(gi << 6);
+            mul_minus_i(a, b, digits(lo64(p) - di), digits(hi64(p) + dr), dr, di);
+            o[0] = make_int4(a.h, a.l, b.h, b.l);
+            if (r >= Kr) put64(o + 2 * kLanes, dr, di);
+            if (T > 1) {   // H: product of the segment's gamma
+                if (r == 0) {
+                    hr = a;
+                    hi = b;
+                } else {
+                    const int64_t x = mul2_fix(a, hr, negative(b), hi), y = mul2_fix(a, hi, b, hr);
+                    hr = digits(x);
+                    hi = digits(y);
+                }
+            }
+            o += 3 * kLanes;
+        }
+        edge[col].dr = dr;
+        edge[col].di = di;
+        edge[col].hr = hr;
+        edge[col].hi = hi;
+    }
+    __syncthreads();
+    // D entering the segment, D of its first Kr rows again, Y of those rows from zero
+    if (on) {
+        int64_t dr = 0, di = 0;
+        for (int k = min(T, sg); k >= 1; --k) {
+            const FixEdge& e = edge[col - k * I];
+            const Digits a = digits(dr), b = digits(di);
+            const int64_t x = mul2_fix(e.hr, a, negative(e.hi), b, e.dr), y = mul2_fix(e.hr, b, e.hi, a, e.di);
+            dr = x;
+            di = y;
+        }
+        int4* o = own;
+        int4 gn = o[0], pn = o[kLanes];
+        for (int r = 0; r < Kr; ++r) {
+            const int4 g = gn, p = pn;
+            if (r + 1 < Kr) {
+                gn = o[3 * kLanes];
+                pn = o[4 * kLanes];
+            }
+            Digits a, b;
+            gam(g, a, b);
+            mul_minus_i(a, b, digits(lo64(p) - di), digits(hi64(p) + dr), dr, di);
+            put64(o + 2 * kLanes, dr, di);
+            o += 3 * kLanes;
+        }
+        int64_t yr = 0, yi = 0;
+        o -= 3 * kLanes;
+        gn = o[0];
+        pn = o[2 * kLanes];
+        for (int r = Kr - 1; r >= 0; --r) {
+            const int4 g = gn, d = pn;
+            if (r > 0) {
+                gn = o[-3 * kLanes];
+                pn = o[-kLanes];
+            }
+            Digits a, b;
+            gam(g, a, b);
+            const Digits u = digits(yr), v = digits(yi);
+            yr = mul2_fix(a, u, negative(b), v, lo64(d));
+            yi = mul2_fix(a, v, b, u, hi64(d));
+            o -= 3 * kLanes;
+        }
+        edge[col].yr = yr;
+        edge[col].yi = yi;
+    }
+    __syncthreads();
+    y_in_r = y_in_i = 0;
+    if (on) {
+        int64_t yr = 0, yi = 0;
+        for (int k = min(T, n_seg - 1 - sg); k >= 1; --k) {
+            const FixEdge& e = edge[col + k * I];
+            const Digits a = digits(yr), b = digits(yi);
+            const int64_t x = mul2_fix(e.hr, a, negative(e.hi), b, e.yr), y = mul2_fix(e.hr, b, e.hi, a, e.yi);
+            yr = x;
+            yi = y;
+        }
+        y_in_r = yr;
+        y_in_i = yi;
+    }
+}
+
 template <bool kCkpt>
 __device__ __forceinline__ bool fix_short_slice(const GroupDesc& G, const ClassDesc& C, const double* __restrict__ tab,
                                                 double2* __restrict__ ps, int64_t nt, int64_t row, int64_t slot, int64_t n0,
@@ -387,14 +532,13 @@ __device__ __forceinline__ bool fix_short_slice(const GroupDesc& G, const ClassD
     const FixClass& F = C.fix;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, P = blockDim.x >> 5;
     const int I = G.I, i = lane & (I - 1), q = lane / I;
-    const int N = G.N, K = G.K, m = G.m, Kg = (K + 1) / 2, Kr = min(m, K), T = (K + m - 1) / m;
+    const int N = G.N, K = G.K, m = G.m;
     const bool on = w < G.P;
     const int sg = w * (kLanes / I) + q, n_seg = G.P * (kLanes / I);   // this lane's segment
     const int s = sg * m, col = w * kLanes + lane;
     const int s_own = on ? min(N, s) : N, e_own = on ? min(N, s + m) : N;
     const bool live = nt > n0;
     const double dx = C.dx;
-    const int4* __restrict__ tT = reinterpret_cast<const int4*>(tab + tab_fxp(C));
     const int4* __restrict__ tO = reinterpret_cast<const int4*>(tab + tab_fob(C));
     auto field = [&](int64_t n) { return n <= nt ? E[row + n - sample_base] : 0.0; };
     int sigma;
@@ -402,20 +546,10 @@ __device__ __forceinline__ bool fix_short_slice(const GroupDesc& G, const ClassD
     if (initial) fix_initial<kCkpt>(G, C, tab, ps, nt, row, s_own, e_own, E, d_out, a_out, sample_base, red, ck);
 
     const double unit = __hiloint2double((1023 + 60 - 2 * sigma) << 20, 0);   // |sigma| <= 112
-    const int64_t inv_b = F.inv_b;
     const int32_t ci = F.ci;
     const Digits cf = F.cf;
     int4* __restrict__ own = buf + (int64_t)w * m * (3 * kLanes) + lane;   // row r: gamma, psi, D at own + r * 96 + (0, 32, 64)
-    auto put64 = [](int4* p, int64_t a, int64_t b) {
-        *p = make_int4((int)(uint32_t)(uint64_t)a, (int)(uint32_t)((uint64_t)a >> 32), (int)(uint32_t)(uint64_t)b,
-                       (int)(uint32_t)((uint64_t)b >> 32));
-    };
-    auto lo64 = [](const int4& v) { return (int64_t)(((uint64_t)(uint32_t)v.y << 32) | (uint32_t)v.x); };
-    auto hi64 = [](const int4& v) { return (int64_t)(((uint64_t)(uint32_t)v.w << 32) | (uint32_t)v.z); };
-    auto gam = [](const int4& v, Digits& r, Digits& m_) {
-        r = Digits{v.x, v.y};
-        m_ = Digits{v.z, v.w};
-    };
+    const ShortGeom geo{N, K, m, I, s, sg, n_seg, col, on, own, edge, reinterpret_cast<const int4*>(tab + tab_fxp(C)), F.inv_b};
     if (on)
         for (int r = 0; r < m; ++r) {
             const int j = s + r;
@@ -423,7 +557,6 @@ __device__ __forceinline__ bool fix_short_slice(const GroupDesc& G, const ClassD
             put64(own + r * (3 * kLanes) + kLanes, double_to_fix((uint64_t)__double_as_longlong(p.x), sigma),
                   double_to_fix((uint64_t)__double_as_longlong(p.y), sigma));
         }
-    auto table = [&](int j) { return __ldg(tT + min(max(j, 0), N - 1)); };
 
     for (int64_t n = n0; n < n1; ++n) {
         const bool active = n < nt, last = n + 1 == n1;
@@ -434,103 +567,11 @@ __device__ __forceinline__ bool fix_short_slice(const GroupDesc& G, const ClassD
         const bool any_put = __any_sync(0xffffffffu, put) || put_ck;
         const Digits Eb = digits(live && n < nt ? __double2ll_rn(0.5 * (field(n) + field(n + 1)) * F.e_scale) : 0);
 
-        // gamma (lead-in and own rows) and D from zero, ascending
-        if (on) {
-            int64_t gr = 0, gi = 0, dr = 0, di = 0;
-            int4 tn = table(s - Kg);
-            for (int r = -Kg; r < 0; ++r) {
-                const int4 t = tn;
-                tn = table(s + r + 1);
-                gamma_row(inv_b, diag_row(FixPoint{t.x, t.y, t.z, t.w}, Eb), gr, gi);
-                if (s + r < 0) gr = gi = 0;   // (a segment's lead-in never lies beyond the far wall unless it does itself)
-            }
-            Digits hr{0, 0}, hi{0, 0};
-            int4 pn = own[kLanes];
-            int4* o = own;
-            for (int r = 0; r < m; ++r) {
-                const int4 t = tn, p = pn;
-                tn = table(s + r + 1);
-                if (r + 1 < m) pn = o[4 * kLanes];
-                gamma_row(inv_b, diag_row(FixPoint{t.x, t.y, t.z, t.w}, Eb), gr, gi);
-                if (s + r >= N) gr = gi = 0;
-                const Digits a = digits(gr << 6), b = digits(gi << 6);
-                mul_minus_i(a, b, digits(lo64(p) - di), digits(hi64(p) + dr), dr, di);
-                o[0] = make_int4(a.h, a.l, b.h, b.l);
-                if (r >= Kr) put64(o + 2 * kLanes, dr, di);
-                if (T > 1) {   // H: product of the segment's gamma
-                    if (r == 0) {
-                        hr = a;
-                        hi = b;
-                    } else {
-                        const int64_t x = mul2_fix(a, hr, negative(b), hi), y = mul2_fix(a, hi, b, hr);
-                        hr = digits(x);
-                        hi = digits(y);
-                    }
-                }
-                o += 3 * kLanes;
-            }
-            edge[col].dr = dr;
-            edge[col].di = di;
-            edge[col].hr = hr;
-            edge[col].hi = hi;
-        }
-        __syncthreads();
-        // D entering the segment, D of its first Kr rows again, Y of those rows from zero
-        if (on) {
-            int64_t dr = 0, di = 0;
-            for (int k = min(T, sg); k >= 1; --k) {
-                const FixEdge& e = edge[col - k * I];
-                const Digits a = digits(dr), b = digits(di);
-                const int64_t x = mul2_fix(e.hr, a, negative(e.hi), b, e.dr), y = mul2_fix(e.hr, b, e.hi, a, e.di);
-                dr = x;
-                di = y;
-            }
-            int4* o = own;
-            int4 gn = o[0], pn = o[kLanes];
-            for (int r = 0; r < Kr; ++r) {
-                const int4 g = gn, p = pn;
-                if (r + 1 < Kr) {
-                    gn = o[3 * kLanes];
-                    pn = o[4 * kLanes];
-                }
-                Digits a, b;
-                gam(g, a, b);
-                mul_minus_i(a, b, digits(lo64(p) - di), digits(hi64(p) + dr), dr, di);
-                put64(o + 2 * kLanes, dr, di);
-                o += 3 * kLanes;
-            }
-            int64_t yr = 0, yi = 0;
-            o -= 3 * kLanes;
-            gn = o[0];
-            pn = o[2 * kLanes];
-            for (int r = Kr - 1; r >= 0; --r) {
-                const int4 g = gn, d = pn;
-                if (r > 0) {
-                    gn = o[-3 * kLanes];
-                    pn = o[-kLanes];
-                }
-                Digits a, b;
-                gam(g, a, b);
-                const Digits u = digits(yr), v = digits(yi);
-                yr = mul2_fix(a, u, negative(b), v, lo64(d));
-                yi = mul2_fix(a, v, b, u, hi64(d));
-                o -= 3 * kLanes;
-            }
-            edge[col].yr = yr;
-            edge[col].yi = yi;
-        }
-        __syncthreads();
-        // Y entering the segment, then the whole segment, descending: psi^{n+1} and the observables
+        int64_t yr, yi;
+        short_solve(geo, Eb, yr, yi);
+        // the whole segment, descending: psi^{n+1} and the observables
         ObsSums ob_sum{0.0, 0.0, 0.0};
         if (on) {
-            int64_t yr = 0, yi = 0;
-            for (int k = min(T, n_seg - 1 - sg); k >= 1; --k) {
-                const FixEdge& e = edge[col + k * I];
-                const Digits a = digits(yr), b = digits(yi);
-                const int64_t x = mul2_fix(e.hr, a, negative(e.hi), b, e.yr), y = mul2_fix(e.hr, b, e.hi, a, e.yi);
-                yr = x;
-                yi = y;
-            }
             int64_t sn = 0, sxh = 0, sxl = 0, svh = 0, svm = 0;
             int4* o = own + (int64_t)(m - 1) * (3 * kLanes);
             int4 gn = o[0], pn = o[kLanes], dn = o[2 * kLanes];
@@ -544,11 +585,7 @@ __device__ __forceinline__ bool fix_short_slice(const GroupDesc& G, const ClassD
                     dn = o[-kLanes];
                     obn = __ldg(tO + min(j - 1, N - 1));
                 }
-                Digits a, b;
-                gam(g, a, b);
-                const Digits u = digits(yr), v = digits(yi);
-                yr = mul2_fix(a, u, negative(b), v, lo64(d));
-                yi = mul2_fix(a, v, b, u, hi64(d));
+                back_row(g, d, yr, yi);
                 int64_t xr = update_fix(ci, cf, digits(yr), lo64(p)), xi = update_fix(ci, cf, digits(yi), hi64(p));
                 if (j < jm_lo || j > jm_hi) {
                     const Digits mm{ob.w, ob.z};

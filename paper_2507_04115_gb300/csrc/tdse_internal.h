@@ -333,7 +333,17 @@ cudaError_t launch_adjoint_full_cn(const GroupDesc* d_groups, int64_t n_groups, 
                                    void* d_work, void* d_tape, void* d_scratch, int rows, int n_max, int kc,
                                    const double* E, const double* gd, const double* ga, double* gE, int mask_on,
                                    int* d_busy, int* d_progress, cudaStream_t st, int have_ckpt = 0,
-                                   void* d_gtape = nullptr);
+                                   void* d_gtape = nullptr, int* d_left = nullptr);
+// The same in 64-bit fixed point (tdse_adjoint_fix.cu), for the groups that have that form; d_left[g] becomes 0 for the
+// groups that are left to launch_adjoint_full_cn (given d_left, it serves those alone).  scratch_per_cta: complex
+// doubles of a CTA's scratch, at least adjoint_fix_scratch; kc < n_max (d_work holds two sums per sample of an
+// interval).
+inline int64_t adjoint_fix_scratch(int P, int m) { return (int64_t)P * m * 3 * kLanes; }
+cudaError_t launch_adjoint_fix(const GroupDesc* d_groups, int64_t n_groups, int P, int ctas, const ClassDesc* d_cls,
+                               const double* d_tab, const int64_t* d_slot_row, const int64_t* d_slot_nt, const void* d_psi0,
+                               void* d_lam, void* d_ckpt, const int64_t* d_ckpt_off, void* d_work, void* d_tape, void* d_scratch,
+                               int64_t scratch_per_cta, int n_max, int kc, const double* E, const double* gd, const double* ga,
+                               double* gE, int mask_on, int* d_busy, int* d_progress, int* d_left, cudaStream_t st, int have_ckpt);
 
 // Energy distribution of every instance state (tdse_resolvent.cu): pivots per (class, energy) into
 // d_piv (2 * piv_elems complex doubles, class c at d_piv_off[c], N_c rows of nE rounded up to 32),

@@ -627,6 +627,56 @@ def test_adjoint_matches_oracle_and_finite_differences(env, lanes):
     b1.close()
 
 
+@pytest.mark.parametrize("N,lanes,warps,kc", [(41, 32, 1, 40), (41, 32, 1, 41), (97, 8, 16, 7), (600, 1, 2, 35), (601, 32, 16, 1),
+                                              (1000, 2, 5, 64), (2001, 32, 4, 70)])
+def test_adjoint_fixed_point_edges(env, N, lanes, warps, kc):
+    """The fixed-point adjoint where it can go wrong: intervals of one step, of the whole pulse and the longest that the
+    smallest grid allows, segments of one row and much longer than the halo, odd grids, instances of 0 and 1 steps,
+    states and gradients of any scale, d alone, a alone, no gradient at all; and a field, a gradient and a state
+    outside the fixed-point range, whose groups the FP64 kernel then serves beside the others."""
+    tdse, oracle = env
+    from paper_2507_04115_gb300 import inputs
+    dx, dt, a = 0.2, 0.05, 1.19
+    nt = [70, 0, 33, 1, 70, 69, 70, 50, 70, 36, 70]
+    n = len(nt)
+    scale = np.array([1.0, 1.0, 3e4, 1.0, 2e-7, 1.0, 1.0, 1.0, 1.0, 1.0, 1e-32])
+    gs = np.array([1.0, 1.0, 1e-9, 1.0, 1e20, 1.0, 1.0, 1.0, 1e-45, 1.0, 1.0])
+    rng = np.random.default_rng(N + kc)
+    rows = [inputs.sin2_pulse(k, dt, 0.08, 0.3, 1.0, 0.4 * i) for i, k in enumerate(nt)]
+    if lanes > 2:    # else these would take every group
+        rows[7] = rows[7].copy()
+        rows[7][20:24] = 2 * 16.0 / (2 * dx * dx * 0.5 * (N - 1) * dx)     # |Re Q| beyond 16
+    else:
+        gs[8] = scale[10] = 1.0
+    offs = np.concatenate([[0], np.cumsum(np.array(nt) + 1)])
+    dev = torch.device("cuda", 0)
+    Et = _device_rows(rows, offs, dev)
+    gd, ga = [], []
+    for i in range(n):
+        gd.append(rng.standard_normal(nt[i] + 1) * gs[i] * (i not in (5, 9)))
+        ga.append(rng.standard_normal(nt[i] + 1) * gs[i] * (i not in (6, 9)))
+    gdt, gat = (torch.from_numpy(np.concatenate(v)).to(dev) for v in (gd, ga))
+    b = tdse.Batch([N] * n, dx, a, nt, dt, row_offsets=offs, absorber=(2.0, 0.125), lanes_per_instance=lanes)
+    b.set_launch(warps_per_cta=warps)
+    psi0, _, _ = oracle.ground_state(N, dx, a, **GS_KW)
+    for i in range(n):
+        b.set_psi(i, torch.from_numpy(psi0 * scale[i]).to(dev))
+    m = oracle.mask(N, dx, 2.0, 0.125)
+    got = [b.adjoint(Et, gdt, gat, ckpt_every=kc).cpu().numpy()]
+    d, acc = torch.zeros_like(Et), torch.zeros_like(Et)
+    b.propagate_checkpointed(Et, d, acc, ckpt_every=kc)
+    got.append(b.adjoint_checkpointed(Et, gdt, gat).cpu().numpy())
+    for i in range(n):
+        sl = slice(offs[i], offs[i + 1])
+        ref = oracle.adjoint(psi0, rows[i], dx, dt, a, gd[i] / gs[i], ga[i] / gs[i], mask_values=m)
+        for g in got:
+            if i == 9:
+                assert np.all(g[sl] == 0.0)
+            else:
+                assert _rel(g[sl] / (gs[i] * scale[i] ** 2), ref) < RTOL_SERIES, (i, _rel(g[sl] / (gs[i] * scale[i] ** 2), ref))
+    b.close()
+
+
 @pytest.mark.parametrize("lanes", [1, 4])
 def test_checkpointed_adjoint_equals_adjoint(env, lanes):
     """tdse_adjoint_checkpointed from a recording made by tdse_propagate_checkpointed in two chunks
