@@ -75,12 +75,14 @@ __global__ void k_ed_pivots(const ClassDesc* __restrict__ cls, int n_cls, const 
     double2* Cp = pivC + piv_off[c];
     if (scheme == 0) {
         // in units of the off-diagonal a: v_j = c'_j = 1 / (b_j / a - v_{j-1}), a chain of 8 dependent
-        // instructions a row (they set the time: 128 energies are 4 warps)
+        // instructions a row (they set the time: 128 energies are 4 warps).  b_j / a = 2 dx^2 (E - V_j) - 2 with one
+        // rounding: those of E - (1/dx^2 + V_j) are 1/(2 dx^2) times larger and act as a shift of E, against eps.
+        // Error of P against 80 bits, N = 4096, dx 0.15, eps 0.02: 9.6e-14 with w_j = b_j - a c'_{j-1}, 1.6e-14 here
         const double inv_a = 2.0 * C.dx * C.dx, bi = zi * inv_a;
         double2 v = make_double2(0.0, 0.0);
         double Vn = V[0];
         for (int j = 0; j < N; ++j) {
-            const double br = (zr - (inv_dx2 + Vn)) * inv_a;
+            const double br = fma(inv_a, zr - Vn, -2.0);
             if (j + 1 < N) Vn = V[j + 1];
             v = cinv(make_double2(br - v.x, bi - v.y));
             Cp[(int64_t)j * nE_pad + k] = v;
