@@ -1333,11 +1333,12 @@ tdse_status tdse_spectrum(const double* a_dev, const int64_t* offsets_host, int6
         longest = std::max(longest, L);
     }
     int B = 0, P = 0;
-    if (shortest > 0 && longest < (int64_t(1) << 30) && 2 * (k_end - 1) < shortest &&
+    if (shortest > 0 && longest < (int64_t(1) << 30) && 2 * (k_end - 1) < shortest && band_dft_allowed(st) &&
         dft_plan(shortest, 2.0 * 3.14159265358979323846 * (double)(k_end - 1) / (double)shortest, k_end - k_begin, &B, &P)) {
-        TDSE_CUDA(launch_band_dft(a_dev, offsets_host, n_rows, dt, nullptr, k_begin, k_end - k_begin, B, P, nullptr, S_dev, st),
-                  "tdse_spectrum");
-        return TDSE_OK;
+        const cudaError_t eb = launch_band_dft(a_dev, offsets_host, n_rows, dt, nullptr, k_begin, k_end - k_begin, B, P, nullptr, S_dev, st);
+        if (eb == cudaSuccess) return TDSE_OK;
+        if (eb != cudaErrorMemoryAllocation) return cuda_fail(eb, "tdse_spectrum");
+        cudaGetLastError();   // no room for the moments: the direct sums
     }
     int64_t* d_off = nullptr;
     TDSE_CUDA(cudaMallocAsync(reinterpret_cast<void**>(&d_off), sizeof(int64_t) * (n_rows + 1), st), "cudaMallocAsync(offsets)");

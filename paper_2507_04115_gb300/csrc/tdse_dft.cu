@@ -20,7 +20,7 @@
 // B and P come from dft_plan, which minimises the instruction count L (P/2 + 1) + n_w (L / B)(P + 6) over
 // them.  Measured, 512 rows of 55160 samples, 400 bins: 170 ms by the direct sum, 4.1 ms here (B = 512,
 // P = 40); both kernels are bound by the FP64 pipe.  The direct sum stays where the band is too wide for
-// blocks or has too few frequencies.
+// blocks or has too few frequencies, on a capturing stream, and without room for the moments.
 #include "tdse_internal.h"
 
 #include <algorithm>
@@ -304,6 +304,12 @@ bool dft_plan(int64_t samples, double turn, int64_t n_w, int* B_out, int* P_out)
     *B_out = best_B;
     *P_out = best_P;
     return best_B > 0;
+}
+
+bool band_dft_allowed(cudaStream_t st)
+{
+    cudaStreamCaptureStatus c = cudaStreamCaptureStatusActive;
+    return cudaStreamIsCapturing(st, &c) == cudaSuccess && c == cudaStreamCaptureStatusNone;
 }
 
 cudaError_t launch_band_dft(const double* a, const int64_t* offs, int64_t n_rows, double dt, const double* omega_host,

@@ -250,9 +250,11 @@ extern "C" tdse_status tdse_dipole_spectrum(const double* a_dev, const int64_t* 
     int64_t longest = 0;
     for (int64_t r = 0; r < n_rows; ++r) longest = std::max(longest, offsets_host[r + 1] - offsets_host[r]);
     int B = 0, P = 0;
-    if (dft_plan(longest, turn, n_omega, &B, &P)) {   // frequencies far below the sampling rate: by block moments
+    if (band_dft_allowed(st) && dft_plan(longest, turn, n_omega, &B, &P)) {   // frequencies far below the sampling rate: by block moments
         const cudaError_t eb = launch_band_dft(a_dev, offsets_host, n_rows, dt, omega_host, 0, n_omega, B, P, weight_dev, out_dev, st);
-        return eb == cudaSuccess ? TDSE_OK : cuda_error(eb, "tdse_dipole_spectrum");
+        if (eb == cudaSuccess) return TDSE_OK;
+        if (eb != cudaErrorMemoryAllocation) return cuda_error(eb, "tdse_dipole_spectrum");
+        cudaGetLastError();   // no room for the moments: the direct sums
     }
     int64_t* d_off = nullptr;
     double* d_om = nullptr;
