@@ -42,12 +42,17 @@ METRIC = "1D-TDSE grid-point-steps/s (batched) & % pipe roofline; mixed vs FP64 
 UNIT = "grid-point-steps/s"
 FLOPS_PER_POINT_STEP = 48.0          # algorithmic FULL_CN work per grid-point step (FMA = 2 flops)
 MIXED_FP64_FLOPS_PER_POINT_STEP = 10.0   # MIXED: the FP64 pivot recurrence per grid-point step
+# FP64 FULL_CN runs in 64-bit fixed point: 32 x 32 -> 64-bit integer multiply-adds of one point and step (pivot and
+# reciprocal 20, the D recurrence twice 28, back substitution 14, update 12, observables 11) on a pipe that takes 16
+# lanes a clock and sub-partition
+MADS_PER_POINT_STEP = 85.0
+MADS_PER_CLK_PER_SM = 64.0
 FP64_FMA_PER_CLK_PER_SM = 2.0        # GB300 FP64 pipe: 2 FMA/clk/SM (1.2 TFLOP/s measured at 2.0 GHz)
 SM_COUNT = 152
 SM_MAX_MHZ = 2070.0
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "k_propagate_full_cn_fp64_volume_traffic.txt")
 KERNEL_SRCS = [os.path.join(ROOT, "paper_2507_04115_gb300", "csrc", f)
-               for f in ("tdse_full_cn.cu", "tdse_sched.cuh", "tdse_device.cuh")]
+               for f in ("tdse_full_cn.cu", "tdse_cn_fix.cuh", "tdse_fix.cuh", "tdse_sched.cuh", "tdse_device.cuh")]
 
 
 def parse_args():
@@ -542,20 +547,29 @@ def own_arm(args):
 
     avg_launch_s = statistics.mean(launch_ms) * 1e-3
     pts_per_launch = float(n) * N * (timed_steps / args.steps)
-    # FP64 work per point-step: the whole step in FP64; in MIXED only the pivot recurrence of the
-    # elimination stays on the FP64 pipe (10 flops + the reciprocal)
-    fp64_flops = FLOPS_PER_POINT_STEP if main_prec == tdse.TDSE_FP64 else MIXED_FP64_FLOPS_PER_POINT_STEP
-    achieved = fp64_flops * pts_per_launch / avg_launch_s
-    peak = FP64_FMA_PER_CLK_PER_SM * 2 * SM_COUNT * SM_MAX_MHZ * 1e6
+    # FP64: integer multiply-adds of the fixed-point step; MIXED: only the pivot recurrence of the elimination is on
+    # the FP64 pipe (10 flops + the reciprocal)
+    peak = FP64_FMA_PER_CLK_PER_SM * 2 * SM_COUNT * SM_MAX_MHZ * 1e6   # FP64 flops
     tpp = kernel_traffic_per_point_step() if main_prec == tdse.TDSE_FP64 else None
     pipes = tdse.tdse_probe_pipes(local_rank)
-    roofline = {"bound": "alu", "achieved": achieved / 1e12, "peak": peak / 1e12, "unit": "TFLOP/s",
-                "frac": achieved / peak, "traffic": (tpp * pts_per_launch) if tpp is not None else None,
-                "kernel": "k_propagate_full_cn<%s>" % args.precision, "pipe": "fp64",
-                "peak_how": "2 FP64 FMA/clk/SM x 152 SMs x 2 flops x 2070 MHz (unit counts at max clock)",
+    if main_prec == tdse.TDSE_FP64:
+        work, top, unit, pipe = MADS_PER_POINT_STEP, MADS_PER_CLK_PER_SM * SM_COUNT * SM_MAX_MHZ * 1e6, "Tmad/s", "integer multiply-add"
+        peak_how = "64 multiply-adds (32 x 32 + 64 bits) /clk/SM x 152 SMs x 2070 MHz (unit counts at max clock)"
+        work_how = "%g integer multiply-adds" % work
+    else:
+        work, top, unit, pipe = MIXED_FP64_FLOPS_PER_POINT_STEP, peak, "TFLOP/s", "fp64"
+        peak_how = "2 FP64 FMA/clk/SM x 152 SMs x 2 flops x 2070 MHz (unit counts at max clock)"
+        work_how = "%g FP64 flops" % work
+    achieved = work * pts_per_launch / avg_launch_s
+    roofline = {"bound": "alu", "achieved": achieved / 1e12, "peak": top / 1e12, "unit": unit,
+                "frac": achieved / top, "traffic": (tpp * pts_per_launch) if tpp is not None else None,
+                "kernel": "k_propagate_full_cn<%s>" % args.precision, "pipe": pipe, "peak_how": peak_how,
                 "fp64_fma_measured_tflops": pipes["fp64_fma_tflops"],
-                "achieved_how": "%g FP64 flops per grid-point step x points x steps per launch / mean CUDA-event "
-                                "launch time" % fp64_flops}
+                "achieved_how": "%s per grid-point step x points x steps per launch / mean CUDA-event launch time" % work_how}
+    if main_prec == tdse.TDSE_FP64:
+        flops = FLOPS_PER_POINT_STEP * pts_per_launch / avg_launch_s
+        roofline["algorithmic_flops"] = {"per_point_step": FLOPS_PER_POINT_STEP, "achieved_tflops": flops / 1e12,
+                                         "over_fp64_pipe_peak": flops / peak}
     if mixed is not None:
         # the MIXED kernel against the FP32 pipe (the algorithmic 48 flops), with the share that stays
         # on the FP64 pipe (the pivot recurrence) against the FP64 peak
@@ -730,7 +744,7 @@ def other_workload(args):
         _line("field ingestion samples/s (Sec. 4.2, zero-padded DFT interpolation)", float(n) * n_fine / t,
               "fine samples/s", args, "%d rows x %d coarse samples (dt %g) -> %d samples (dt %g)" % (n, M, dt_c, n_fine, dt_f),
               dict(rows=n, M=M, dt_coarse=dt_c, dt_fine=dt_f, n_fine=n_fine), dtype="f64",
-              fp64_instructions_per_sample=6 * (M // 2 + 1), seconds_per_call=t)
+              fp64_instructions_per_sample=16 + M * (M // 2 + 1) // n_fine, seconds_per_call=t)
         return
 
     if args.workload == "populations":
@@ -1006,7 +1020,7 @@ def measure_field(torch, tdse, inputs, dev, stream, rows=2048, repeats=2):
     t = min(_timed(torch, dev, stream, lambda: tdse.resample_field(coarse, dt_c, dt_f, n_fine, out=out))
             for _ in range(repeats))
     return {"value": float(n) * n_fine / t, "unit": "fine samples/s", "seconds_per_call": t, "rows": n, "M": M,
-            "n_fine": n_fine, "fp64_instructions_per_sample": 6 * (M // 2 + 1)}
+            "n_fine": n_fine, "fp64_instructions_per_sample": 16 + M * (M // 2 + 1) // n_fine}
 
 
 # ------------------------------------------------------------------------------------------- configuration-size runs

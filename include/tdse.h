@@ -58,9 +58,12 @@ typedef enum {
 } tdse_status;
 
 typedef enum {
-    TDSE_FP64 = 0,   /* the solve and the wavefunctions in IEEE double; |psi|^2 and the observable
-                        sums as float pairs (about 2^-44 relative per point) over blocks of 16
-                        points, added in double across blocks */
+    TDSE_FP64 = 0,   /* the wavefunctions in IEEE double between calls; within a call the steps and the
+                        observable sums in 64-bit fixed point (60 bits of an instance's norm, gamma to
+                        2^-58; error not above that of the sweep in double), for dt/(4 dx^2) in [0.0715, 0.35]
+                        (FULL_CN), N <= 32768, usual fields and norms; otherwise, per slice of a group, the
+                        solve in double and |psi|^2 and the sums as float pairs (about 2^-44 relative per
+                        point) over blocks of 16 points, added in double across blocks */
     TDSE_MIXED = 1   /* psi, the solve's right-hand side and back substitution in float; the
                         elimination recurrence (pivots) in double; the observables as float
                         partial sums over 16 points, added in double across blocks */
@@ -147,6 +150,8 @@ tdse_status tdse_copy_state(tdse_batch* batch, void* buffer_dev, int32_t directi
  * psi^0 (call after tdse_ground_state, tdse_set_psi or tdse_copy_state, before propagating), and
  * are left unchanged.  The loss gradients gd_n = dL/dd_n and ga_n = dL/da_n, the field E and the
  * output gE_n = dL/dE_n use the batch's row layout with sample_base 0 and n = 0..Nt_i.
+ * Both sweeps run in 64-bit fixed point where the group's fields, states and gradients are within its range
+ * and ckpt_every is below the largest N, otherwise in double.
  *   ckpt_every  states are checkpointed every ckpt_every steps and recomputed in between (one
  *               interval of states is kept per CTA); memory ~ (Nt/ckpt_every + ckpt_every) states.
  * With lambda^n = 2 dL/d conj(psi^n): lambda^Nt = g^Nt; mu = B_n^{-1} M lambda^{n+1};
@@ -240,8 +245,8 @@ tdse_status tdse_populations(tdse_batch* batch, double r_core, double* out_dev, 
  * ends of the padded spectrum), else 1 -- the trigonometric interpolant, which reproduces the coarse
  * samples exactly.  It is T-periodic: times beyond the window wrap around, so pad the coarse row
  * with zeros past the pulse.  With out_stride equal to a batch's row stride the output feeds
- * tdse_propagate directly.  M in [2, 8192]; computed in FP64; synchronous (allocates
- * n_rows x (M/2+1) x 16 bytes for the call). */
+ * tdse_propagate directly.  M in [2, 8192]; computed in FP64; synchronous (allocates coefficients and
+ * transform nodes for a bounded number of rows and 132 bytes per output sample for the call). */
 tdse_status tdse_resample_field(const double* coarse_dev, int64_t n_rows, int32_t M, double dt_coarse, double dt_fine,
                                 int64_t n_fine, int64_t out_stride, double* out_dev, int device, void* stream);
 
@@ -254,7 +259,8 @@ tdse_status tdse_resample_field(const double* coarse_dev, int64_t n_rows, int32_
  *   omega_host     n_omega angular frequencies (same time unit as dt; |omega| <= 1e6)
  *   weight_dev     NULL (weight 1) or device n_rows doubles: the gas density of each row's point
  *   out_dev        device, n_rows x n_omega complex values as (re, im) double pairs, row-major
- * FP64.  Asynchronous on the stream (stream-ordered allocation of the offsets and frequencies).
+ * FP64.  Asynchronous on the stream (stream-ordered allocation of the offsets and frequencies, and of up to
+ * 256 MB, or one row's share if that is more, for block moments where the frequencies allow them).
  * The rows of a volume laid out radius-major (row = i_rho * n_z + i_z) give the source layout of
  * tdse_hankel directly. */
 tdse_status tdse_dipole_spectrum(const double* a_dev, const int64_t* offsets_host, int64_t n_rows, double dt,
@@ -329,9 +335,11 @@ tdse_status tdse_plan(const tdse_batch* batch, tdse_plan_info* info_host);
 tdse_status tdse_set_layout(tdse_batch* batch, int32_t lanes_per_instance);
 
 /* Override the launch configuration for later calls (0 keeps the default of each):
- * warps_per_cta in [1, 16] (default 8 for FP64, 12 for MIXED FULL_CN, 16 for MIXED NUMEROV_SPLIT; also
- * the largest number of segments per instance),
- * ctas_per_sm in [1, 32] (default 1; clamped to the occupancy limit), slice_steps >= 1 (default 16),
+ * warps_per_cta in [1, 16] (default: FP64 by the estimated cost of a step, up to 16 / ctas_per_sm, or 8 where
+ * no class has the fixed-point form; 12 for MIXED FULL_CN, 16 for MIXED NUMEROV_SPLIT; also the largest number
+ * of segments per instance),
+ * ctas_per_sm in [1, 32] (default 1; FP64 1, 2 or 4 by the estimated makespan; clamped to the occupancy limit),
+ * slice_steps >= 1 (default 16),
  * max_ctas >= 1 caps the persistent grid (default: no cap beyond SMs x ctas_per_sm and the number
  * of groups).  Synchronises the device; the scratch is reallocated. */
 tdse_status tdse_set_launch(tdse_batch* batch, int32_t warps_per_cta, int32_t ctas_per_sm, int32_t slice_steps,

@@ -12,6 +12,10 @@
 //             to E_{n+1}; dL/dE_n += ga_n dx sum_j |psi^n_j|^2 (the E_n in a_n)
 // The solve with A_n reuses the forward kernel's segmented, halo-truncated Thomas sweep.
 //
+// Groups within the fixed-point range are served by tdse_adjoint_fix.cu (44.4 -> 14.7 ms at 1024 x 2048 points, 96
+// steps); this kernel runs behind it for the others, or alone when no class has that form or the checkpoint
+// interval is as long as the largest grid.
+//
 // Memory: the forward states are recomputed from checkpoints every K steps; within a checkpoint
 // interval the pre-mask states psi~ are kept on a per-CTA tape.  One CTA owns a group for the whole
 // call: first a forward pass writing the checkpoints (unless a checkpointed forward propagation has

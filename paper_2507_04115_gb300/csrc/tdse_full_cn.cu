@@ -23,6 +23,10 @@
 //     (8192 instances = 256 groups on 152 SMs) and when groups have different lengths.
 // HBM layouts: psi [group][j][lane] (16 B per point, a warp reads 512 contiguous bytes), scratch per
 // CTA [warp][row][gamma | D][lane].
+//
+// FP64 slices whose class, fields and states are within the fixed-point range run on the integer pipe
+// (tdse_cn_fix.cuh: 2.7 times the rate on the volume batch, 6.5 on one atom); the FP64 sweeps here serve the others
+// and MIXED.
 #include "tdse_cn_fix.cuh"
 
 namespace tdse {

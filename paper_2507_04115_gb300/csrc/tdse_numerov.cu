@@ -1,6 +1,7 @@
 // NUMEROV_SPLIT real-time propagation kernel of libtdse (sm_103a), FP64 and MIXED precision.  It
 // shares the lane-batched layout, the halo-segmented sweeps and the persistent group scheduler of
-// the FULL_CN kernel (see tdse_full_cn.cu).
+// the FULL_CN kernel (see tdse_full_cn.cu).  FP64 slices within the fixed-point range run on the integer pipe
+// (tdse_numerov_fix.cuh); the FP64 sweeps here serve the others and MIXED.
 #include "tdse_numerov_fix.cuh"
 
 namespace tdse {
