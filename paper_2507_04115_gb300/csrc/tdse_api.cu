@@ -1196,7 +1196,7 @@ tdse_status tdse_energy_distribution(tdse_batch* b, const double* E_grid_host, i
         piv_elems += (int64_t)b->classes[c].N * nE_pad;
         n_max = std::max(n_max, b->classes[c].N);
     }
-    const int64_t sc = energy_distribution_scratch_elems(b->sm_count, n_max);
+    const int64_t sc = energy_distribution_scratch_elems(b->sm_count, n_max, (int)b->scheme, b->n_slots, n_energies);
     if (sc > b->ed_scratch_elems) {
         TDSE_CUDA(cudaStreamSynchronize(st), "tdse_energy_distribution: synchronize");
         cudaFree(b->d_ed_scratch);

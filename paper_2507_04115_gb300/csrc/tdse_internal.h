@@ -348,7 +348,7 @@ cudaError_t launch_adjoint_fix(const GroupDesc* d_groups, int64_t n_groups, int 
 // Energy distribution of every instance state (tdse_resolvent.cu): pivots per (class, energy) into
 // d_piv (2 * piv_elems complex doubles, class c at d_piv_off[c], N_c rows of nE rounded up to 32),
 // then one warp per (instance, 32 energies) with a scratch of energy_distribution_scratch_elems.
-int64_t energy_distribution_scratch_elems(int sm_count, int n_max);
+int64_t energy_distribution_scratch_elems(int sm_count, int n_max, int scheme, int64_t n_slots, int nE);
 cudaError_t launch_energy_distribution(int mixed, const GroupDesc* d_groups, const ClassDesc* d_cls, int n_cls,
                                        const double* d_tab, const int64_t* d_slot_group, const int64_t* d_slot_inst,
                                        int64_t n_slots, const void* d_psi, const double* d_E_grid, int nE, double eps,

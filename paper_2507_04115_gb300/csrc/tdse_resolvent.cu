@@ -115,10 +115,11 @@ __global__ void k_ed_solve(const GroupDesc* __restrict__ groups, const ClassDesc
 {
     constexpr int scheme = kScheme;
     const int lane = threadIdx.x & 31;
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t n_warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     const int nkb = nE_pad / kLanes;
-    double2* __restrict__ sc = scratch + warp * (int64_t)n_max * kLanes;
+    const int64_t warp = n_slots * nkb < n_warps ? (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x
+                                                 : ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    double2* __restrict__ sc = scratch + warp * (int64_t)n_max * kLanes;   // (touched with a task only: warp < tasks)
     for (int64_t task = warp; task < n_slots * nkb; task += n_warps) {
         const int64_t slot = task / nkb;
         const int kb = (int)(task % nkb);
@@ -238,16 +239,20 @@ cudaError_t launch_ionisation(const double* d_P, int64_t n_inst, int nE, const d
     return cudaGetLastError();
 }
 
-// Warps per SM: a warp's two dependent sweeps leave the FP64 pipe idle for half of the time at 8 warps; 16
-// while their scratch stays below 8 GB.
-static int solve_warps(int sm_count, int n_max)
+// Blocks of 8 warps, one warp per task (slot, 32 energies) at a time.  FULL_CN: 2 an SM, as a warp's two dependent sweeps
+// leave the FP64 pipe idle for half of the time with one, while their scratch stays below 8 GB; the Numerov pencil, whose
+// rows have more independent work, gained 0.5 % from it (8.15 and 8.11 ms): 1.  Fewer tasks than warps: spread over the
+// blocks, and no more scratch (which the first call allocates) than tasks.
+static int solve_blocks(int sm_count, int n_max, int scheme, int64_t tasks)
 {
-    return (int64_t)sm_count * 16 * kLanes * n_max * (int64_t)sizeof(double2) <= (int64_t(8) << 30) ? 16 : 8;
+    const bool two = scheme == 0 && (int64_t)sm_count * 16 * kLanes * n_max * (int64_t)sizeof(double2) <= (int64_t(8) << 30);
+    return (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)sm_count * (two ? 2 : 1), tasks));
 }
 
-int64_t energy_distribution_scratch_elems(int sm_count, int n_max)
+int64_t energy_distribution_scratch_elems(int sm_count, int n_max, int scheme, int64_t n_slots, int nE)
 {
-    return (int64_t)sm_count * solve_warps(sm_count, n_max) * kLanes * n_max;
+    const int64_t tasks = n_slots * ((nE + kLanes - 1) / kLanes);
+    return std::max<int64_t>(1, std::min<int64_t>((int64_t)solve_blocks(sm_count, n_max, scheme, tasks) * 8, tasks)) * kLanes * n_max;
 }
 
 cudaError_t launch_energy_distribution(int mixed, const GroupDesc* d_groups, const ClassDesc* d_cls, int n_cls,
@@ -264,7 +269,7 @@ cudaError_t launch_energy_distribution(int mixed, const GroupDesc* d_groups, con
     k_ed_pivots<<<pg, 128, 0, st>>>(d_cls, n_cls, d_tab, d_E_grid, nE, nE_pad, eps, scheme, pivW, pivC, d_piv_off);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const int blocks = sm_count * (solve_warps(sm_count, n_max) / 8);   // of 8 warps, as the scratch holds
+    const int blocks = solve_blocks(sm_count, n_max, scheme, n_slots * (nE_pad / kLanes));
     auto solve = [&](auto kernel, auto psi) {
         kernel<<<blocks, 256, 0, st>>>(d_groups, d_cls, d_tab, d_slot_group, d_slot_inst, n_slots, psi, d_E_grid, nE, nE_pad, eps,
                                        pivW, pivC, d_piv_off, static_cast<double2*>(d_scratch), n_max, P_out);
