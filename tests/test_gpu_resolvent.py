@@ -60,6 +60,26 @@ def test_energy_distribution_matches_oracle(env, scheme, precision, lanes):
     b.close()
 
 
+@pytest.mark.parametrize("scheme", [0, 1])
+def test_solves_do_not_depend_on_their_number(env, scheme):
+    """More solves than warps in one call, and fewer (spread over the blocks, with scratch for no more) in three
+    calls that the scratch grows between: the same bits, also with the calls in the other order."""
+    tdse, _ = env
+    n, N, nt, dt = 1000, 200, 8, 0.05
+    dev = torch.device("cuda", 0)
+    Et = torch.from_numpy(np.random.default_rng(5).uniform(-0.1, 0.1, n * (nt + 1))).to(dev)
+    b = tdse.Batch([N] * n, 0.2, 1.2, [nt] * n, dt, absorber=(5.0, 0.125), scheme=scheme)
+    b.ground_state(**GS_KW)
+    b.propagate(Et, torch.zeros_like(Et), torch.zeros_like(Et))
+    grid = np.linspace(-0.8, 1.5, 96)
+    parts = torch.cat([b.energy_distribution(grid[k: k + 32], 0.03) for k in (0, 32, 64)], dim=1)
+    one = b.energy_distribution(grid[5:6], 0.03)
+    whole = b.energy_distribution(grid, 0.03)
+    assert torch.equal(whole, parts) and torch.equal(whole[:, 5:6], one)
+    assert torch.equal(b.energy_distribution(grid[:32], 0.03), whole[:, :32])
+    b.close()
+
+
 def test_energy_distribution_of_ground_state_peaks_at_its_energy(env):
     """Right after the ground state the distribution is a Lorentzian at the ground energy: its peak
     value is 1/(pi eps) (norm 1) and half of it at E_g +- eps."""
