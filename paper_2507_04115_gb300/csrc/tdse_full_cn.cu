@@ -257,7 +257,6 @@ k_propagate_full_cn(const GroupDesc* __restrict__ groups, int64_t n_groups, cons
     const int w = threadIdx.x >> 5;
     const int P = blockDim.x >> 5;
     Cx* __restrict__ psi_all = static_cast<Cx*>(psi_raw);
-    Cx* __restrict__ sc = static_cast<Cx*>(scratch_raw) + ((int64_t)blockIdx.x * P + w) * rows * (2 * kLanes);
     // MIXED: per-warp ring of bulk-copy slots after the reduction area (see the back substitution)
     const int kRing = ring_slots;   // bulk-copy slots per warp (MIXED)
     uint64_t* bars = reinterpret_cast<uint64_t*>(red + P * 3 * kLanes) + w * kRing;
@@ -288,10 +287,10 @@ k_propagate_full_cn(const GroupDesc* __restrict__ groups, int64_t n_groups, cons
         __syncthreads();   // s_g / s_k are rewritten only after every warp has read them
         if (g < 0) break;
 
-        const GroupDesc G = groups[g];
+        GroupDesc G = groups[g];
         const ClassDesc C = cls[G.cls];
         const Fma64 F{C.one, C.nzero};
-        const int N = G.N, Pg = G.P, K = G.K, m = G.m;
+        const int N = G.N, K = G.K;
         const int64_t slot = G.slot0 + (lane & (G.I - 1));   // this lane's instance
         const int64_t nt = slot_nt[slot];   // -1 for padding lanes
         const int64_t row = slot_row[slot];
@@ -299,11 +298,6 @@ k_propagate_full_cn(const GroupDesc* __restrict__ groups, int64_t n_groups, cons
         const double inv_beta = 1.0 / beta;
         const R two_over_beta = (R)(2.0 / beta);
         const double dx = C.dx;
-        // warps beyond the group's segment count own an empty segment
-        const int s = w < Pg ? min(N, w * m) : N;
-        const int e = w < Pg ? min(N, s + m) : N;
-        const int lo = w < Pg ? max(0, s - K) : N;
-        const int hi = w < Pg ? min(N, e + K) : N;
         Cx* __restrict__ ps = psi_all + G.psi_off;
         const double2* __restrict__ tab_ab2 = reinterpret_cast<const double2*>(tab + tab_ab(C));
         const double2* __restrict__ tab_xv2 = reinterpret_cast<const double2*>(tab + tab_xv(C));
@@ -327,6 +321,18 @@ k_propagate_full_cn(const GroupDesc* __restrict__ groups, int64_t n_groups, cons
                 done = fix_slice<kCkpt>(G, C, tab, ps, nt, row, slot, n0, n1, kslice == 0 && step_begin == 0, E, d_out, a_out,
                                         sample_base, reinterpret_cast<int4*>(scratch_raw) + (int64_t)blockIdx.x * P * rows * (2 * kLanes),
                                         red, status, kCkpt ? ckpt + ckpt_off[g] : nullptr, kc, jm_lo, jm_hi);
+        Cx* __restrict__ sc = static_cast<Cx*>(scratch_raw) + ((int64_t)blockIdx.x * P + w) * rows * (2 * kLanes);
+        if constexpr (!kMixed) {   // the FP64 sweeps' own split, packed into the CTA's scratch
+            G.P = G.P64;
+            G.m = G.m64;
+            sc = static_cast<Cx*>(scratch_raw) + ((int64_t)blockIdx.x * P * rows + (int64_t)w * (G.m + 2 * K)) * (2 * kLanes);
+        }
+        // warps beyond the group's segment count own an empty segment
+        const int Pg = G.P, m = G.m;
+        const int s = w < Pg ? min(N, w * m) : N;
+        const int e = w < Pg ? min(N, s + m) : N;
+        const int lo = w < Pg ? max(0, s - K) : N;
+        const int hi = w < Pg ? min(N, e + K) : N;
         if (done) {
         } else if (G.I != kLanes) {
             split_slice<kMixed, kCkpt>(G, F, ps, tab_ab2, tab_xv2, tab_m, inv_beta, two_over_beta, dx, jm_lo, jm_hi,

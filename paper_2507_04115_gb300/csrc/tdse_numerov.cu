@@ -236,9 +236,6 @@ k_propagate_numerov(const GroupDesc* __restrict__ groups, int64_t n_groups, cons
     const int w = threadIdx.x >> 5;
     const int P = blockDim.x >> 5;
     Cx* __restrict__ psi_all = static_cast<Cx*>(psi_raw);
-    // scratch rows: d_j only (one complex per row per lane)
-    Cx* __restrict__ sc = static_cast<Cx*>(scratch_raw) + ((int64_t)blockIdx.x * P + w) * rows * (2 * kLanes);
-
     for (;;) {
         if (w == 0) {
             int k = 0;
@@ -255,18 +252,14 @@ k_propagate_numerov(const GroupDesc* __restrict__ groups, int64_t n_groups, cons
         __syncthreads();
         if (g < 0) break;
 
-        const GroupDesc G = groups[g];
+        GroupDesc G = groups[g];
         const ClassDesc C = cls[G.cls];
         const Fma64 F{C.one, C.nzero};
-        const int N = G.N, Pg = G.P, K = G.K, m = G.m;
+        const int N = G.N, K = G.K;
         const int64_t slot = G.slot0 + (lane & (G.I - 1));   // this lane's instance
         const int64_t nt = slot_nt[slot];
         const int64_t row = slot_row[slot];
         const double dx = C.dx;
-        const int s = w < Pg ? min(N, w * m) : N;
-        const int e = w < Pg ? min(N, s + m) : N;
-        const int lo = w < Pg ? max(0, s - K) : N;
-        const int hi = w < Pg ? min(N, e + K) : N;
         Cx* __restrict__ ps = psi_all + G.psi_off;
         const double2* __restrict__ tab_xv2 = reinterpret_cast<const double2*>(tab + tab_xv(C));
         const double* __restrict__ tab_m = tab + tab_mk(C);
@@ -290,6 +283,18 @@ k_propagate_numerov(const GroupDesc* __restrict__ groups, int64_t n_groups, cons
                                          a_out, sample_base,
                                          reinterpret_cast<int4*>(scratch_raw) + (int64_t)blockIdx.x * P * rows * (2 * kLanes),
                                          red, status, jm_lo, jm_hi);
+        // scratch rows: d_j only (one complex per row per lane)
+        Cx* __restrict__ sc = static_cast<Cx*>(scratch_raw) + ((int64_t)blockIdx.x * P + w) * rows * (2 * kLanes);
+        if constexpr (!kMixed) {   // the FP64 sweeps' own split, packed into the CTA's scratch
+            G.P = G.P64;
+            G.m = G.m64;
+            sc = static_cast<Cx*>(scratch_raw) + ((int64_t)blockIdx.x * P * rows + (int64_t)w * (G.m + 2 * K)) * (2 * kLanes);
+        }
+        const int Pg = G.P, m = G.m;
+        const int s = w < Pg ? min(N, w * m) : N;
+        const int e = w < Pg ? min(N, s + m) : N;
+        const int lo = w < Pg ? max(0, s - K) : N;
+        const int hi = w < Pg ? min(N, e + K) : N;
         if (done) {
         } else if (G.I != kLanes) {
             numerov_split_slice<kMixed>(G, C, F, ps, tW, tL, tC, tF, tab_xv2, tab_m, jm_lo, jm_hi, nt, row, slot, n0,

@@ -65,6 +65,8 @@ __global__ void k_static_setup(ClassDesc C, int64_t n_inst, int64_t n_groups, in
         G.P = P;
         G.K = K;
         G.m = m;
+        G.P64 = P;
+        G.m64 = m;
         G.I = kLanes;
         G.w = 1;
         groups[g] = G;
