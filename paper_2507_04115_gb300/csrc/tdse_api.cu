@@ -130,6 +130,7 @@ struct tdse_batch {
     size_t gtape_bytes = 0;
     bool use_gtape = true;             // tdse_set_adjoint_gamma_tape
     int adj_kc = 0, adj_ctas = 0;
+    bool any_fix = false;              // a class of the batch has the fixed-point form
     // launch shape of the adjoint kernels (one CTA per SM: the fixed-point rules where a class has that form)
     std::vector<GroupDesc> adj_groups;
     GroupDesc* d_adj_groups = nullptr;
@@ -541,6 +542,7 @@ tdse_status build_plan(tdse_batch* b)
     b->slice = b->slice_override > 0 ? b->slice_override : 16;
     bool fix = false;
     for (const ClassDesc& C : b->classes) fix = fix || on_fix_path(b, C);
+    b->any_fix = fix;
     int want = 1;
     if (b->ctas_per_sm_override > 0)
         want = b->ctas_per_sm_override;
@@ -558,7 +560,7 @@ tdse_status build_plan(tdse_batch* b)
         b->class_P[G.cls] = std::max(b->class_P[G.cls], G.P);
         b->class_K[G.cls] = std::max(b->class_K[G.cls], G.K);
     }
-    const int per_sm_max = propagate_max_ctas_per_sm(b->mixed(), b->warps);
+    const int per_sm_max = propagate_max_ctas_per_sm(b->mixed(), fix, b->warps);
     const int per_sm = std::min(want, per_sm_max);
     b->ring = propagate_ring_slots(b->warps, per_sm);
     auto grid = [&](int k) {
@@ -571,7 +573,7 @@ tdse_status build_plan(tdse_batch* b)
         // the adjoint kernels' shape; they share the scratch
         b->adj_groups = b->groups;
         b->adj_rows = shape_groups(b, b->adj_groups, fix, 1, &b->adj_warps);
-        b->adj_grid = grid(b->ctas_per_sm_override > 0 ? std::min(b->ctas_per_sm_override, propagate_max_ctas_per_sm(0, b->adj_warps)) : 1);
+        b->adj_grid = grid(b->ctas_per_sm_override > 0 ? std::min(b->ctas_per_sm_override, propagate_max_ctas_per_sm(0, fix, b->adj_warps)) : 1);
         sc = std::max(sc, (int64_t)b->adj_grid * b->adj_warps * b->adj_rows * 2 * kLanes);
         b->adj_fix_scratch = 0;
         for (const GroupDesc& G : b->adj_groups)
@@ -1001,13 +1003,13 @@ static tdse_status propagate_impl(tdse_batch* b, const double* E_dev, double* d_
     if (!guard.ok) return fail(TDSE_ERR_CUDA, "cudaSetDevice failed");
     cudaStream_t st = (cudaStream_t)stream;
     if (b->scheme == TDSE_NUMEROV_SPLIT)
-        TDSE_CUDA(launch_propagate_numerov(b->mixed(), b->d_groups, (int64_t)b->groups.size(), b->warps, b->ctas,
+        TDSE_CUDA(launch_propagate_numerov(b->mixed(), b->any_fix, b->d_groups, (int64_t)b->groups.size(), b->warps, b->ctas,
                                            b->d_cls, b->d_tab, b->d_slot_row, b->d_slot_nt, b->d_psi, b->d_scratch,
                                            b->rows, E_dev, d_dev, a_dev, sample_base, step_begin, step_end, b->slice,
                                            b->mask_on, b->dt, b->d_busy, b->d_progress, b->d_status, st),
                   "propagate launch");
     else
-        TDSE_CUDA(launch_propagate_full_cn(b->mixed(), b->d_groups, (int64_t)b->groups.size(), b->warps, b->ctas,
+        TDSE_CUDA(launch_propagate_full_cn(b->mixed(), b->any_fix, b->d_groups, (int64_t)b->groups.size(), b->warps, b->ctas,
                                            b->d_cls, b->d_tab, b->d_slot_row, b->d_slot_nt, b->d_psi, b->d_scratch,
                                            b->rows, E_dev, d_dev, a_dev, sample_base, step_begin, step_end, b->slice,
                                            b->mask_on, b->d_busy, b->d_progress, b->d_status, b->ring, b->wait_polls, st,

@@ -239,7 +239,11 @@ __device__ __forceinline__ void fwd_row_f32(float2 t, float2 p, float Eb, float 
     Dr = nDr;
 }
 
-template <bool kMixed, bool kCkpt>
+// kFix: classes with the fixed-point form may be among the groups.  Batches without one run the kernel that holds their
+// sweeps alone: beside the fixed-point forms the compiler's schedule of these is 2.5 to 5 % slower, and the forms' shared
+// memory takes from L1 (64 x 8192 points at 32 lanes, dt / (4 dx^2) = 0.5, 64 steps: 14.64 ms and 14.06; 8192 x 4096
+// points, 32 steps: 71.2 and 69.5).
+template <bool kMixed, bool kCkpt, bool kFix>
 __global__ void __launch_bounds__(512, 1)
 k_propagate_full_cn(const GroupDesc* __restrict__ groups, int64_t n_groups, const ClassDesc* __restrict__ cls,
                     const double* __restrict__ tab, const int64_t* __restrict__ slot_row,
@@ -287,7 +291,7 @@ k_propagate_full_cn(const GroupDesc* __restrict__ groups, int64_t n_groups, cons
         __syncthreads();   // s_g / s_k are rewritten only after every warp has read them
         if (g < 0) break;
 
-        GroupDesc G = groups[g];
+        const GroupDesc G = groups[g];
         const ClassDesc C = cls[G.cls];
         const Fma64 F{C.one, C.nzero};
         const int N = G.N, K = G.K;
@@ -310,7 +314,7 @@ k_propagate_full_cn(const GroupDesc* __restrict__ groups, int64_t n_groups, cons
         const int64_t n1 = min(n_end, n0 + slice);
 
         bool done = false;
-        if constexpr (!kMixed)
+        if constexpr (kFix)
             if (C.fix.ok && fix_short(G))
                 done = fix_short_slice<kCkpt>(G, C, tab, ps, nt, row, slot, n0, n1, kslice == 0 && step_begin == 0, E, d_out,
                                               a_out, sample_base,
@@ -321,21 +325,22 @@ k_propagate_full_cn(const GroupDesc* __restrict__ groups, int64_t n_groups, cons
                 done = fix_slice<kCkpt>(G, C, tab, ps, nt, row, slot, n0, n1, kslice == 0 && step_begin == 0, E, d_out, a_out,
                                         sample_base, reinterpret_cast<int4*>(scratch_raw) + (int64_t)blockIdx.x * P * rows * (2 * kLanes),
                                         red, status, kCkpt ? ckpt + ckpt_off[g] : nullptr, kc, jm_lo, jm_hi);
+        if (!done) {   // (all that the FP64 sweeps need inside: held across the fixed-point forms it slows them by 1 to 7 %)
         Cx* __restrict__ sc = static_cast<Cx*>(scratch_raw) + ((int64_t)blockIdx.x * P + w) * rows * (2 * kLanes);
-        if constexpr (!kMixed) {   // the FP64 sweeps' own split, packed into the CTA's scratch
-            G.P = G.P64;
-            G.m = G.m64;
-            sc = static_cast<Cx*>(scratch_raw) + ((int64_t)blockIdx.x * P * rows + (int64_t)w * (G.m + 2 * K)) * (2 * kLanes);
+        GroupDesc H = G;
+        if constexpr (kFix) {   // the FP64 sweeps' own split, packed into the CTA's scratch
+            H.P = G.P64;
+            H.m = G.m64;
+            sc = static_cast<Cx*>(scratch_raw) + ((int64_t)blockIdx.x * P * rows + (int64_t)w * (H.m + 2 * K)) * (2 * kLanes);
         }
         // warps beyond the group's segment count own an empty segment
-        const int Pg = G.P, m = G.m;
+        const int Pg = H.P, m = H.m;
         const int s = w < Pg ? min(N, w * m) : N;
         const int e = w < Pg ? min(N, s + m) : N;
         const int lo = w < Pg ? max(0, s - K) : N;
         const int hi = w < Pg ? min(N, e + K) : N;
-        if (done) {
-        } else if (G.I != kLanes) {
-            split_slice<kMixed, kCkpt>(G, F, ps, tab_ab2, tab_xv2, tab_m, inv_beta, two_over_beta, dx, jm_lo, jm_hi,
+        if (G.I != kLanes) {
+            split_slice<kMixed, kCkpt>(H, F, ps, tab_ab2, tab_xv2, tab_m, inv_beta, two_over_beta, dx, jm_lo, jm_hi,
                                        nt, row, slot, n0, n1, kslice == 0 && step_begin == 0, E, d_out, a_out,
                                        sample_base, sc, red, status, kCkpt ? ckpt + ckpt_off[g] : nullptr, kc,
                                        reinterpret_cast<const float4*>(tab + (kMixed ? tab_fx(C) : tab_xff(C))));
@@ -674,6 +679,7 @@ k_propagate_full_cn(const GroupDesc* __restrict__ groups, int64_t n_groups, cons
                 }
         }
         }   // 32-wide group
+        }
 
         if (timed_out) status[slot] = 2;   // a bulk copy did not complete in time
 
@@ -689,7 +695,7 @@ k_propagate_full_cn(const GroupDesc* __restrict__ groups, int64_t n_groups, cons
     }
 }
 
-cudaError_t launch_propagate_full_cn(int mixed, const GroupDesc* d_groups, int64_t n_groups, int P, int ctas,
+cudaError_t launch_propagate_full_cn(int mixed, int fix, const GroupDesc* d_groups, int64_t n_groups, int P, int ctas,
                                      const ClassDesc* d_cls, const double* d_tab, const int64_t* d_slot_row,
                                      const int64_t* d_slot_nt, void* d_psi, void* d_scratch, int rows,
                                      const double* E, double* d_out, double* a_out, int64_t sample_base,
@@ -704,48 +710,46 @@ cudaError_t launch_propagate_full_cn(int mixed, const GroupDesc* d_groups, int64
     e = cudaMemsetAsync(d_progress, 0, sizeof(int) * n_groups, st);
     if (e != cudaSuccess) return e;
     if (mixed && (ring < kMinRing || ring > kMaxRing)) return cudaErrorInvalidValue;
-    const size_t smem = full_cn_smem_bytes(mixed, P, ring);
+    const size_t smem = full_cn_smem_bytes(mixed, fix, P, ring);
     if (mixed) {
         static std::atomic<bool> attr_set[kMaxAttrDevices];
         int dev = 0;
         if (attr_needed(attr_set, &dev)) {
-            e = cudaFuncSetAttribute(k_propagate_full_cn<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            e = cudaFuncSetAttribute(k_propagate_full_cn<true, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)full_cn_smem_max_bytes());
             if (e != cudaSuccess) return e;
             attr_done(attr_set, dev);
         }
-        k_propagate_full_cn<true, false><<<(unsigned)ctas, P * kLanes, smem, st>>>(
+        k_propagate_full_cn<true, false, false><<<(unsigned)ctas, P * kLanes, smem, st>>>(
             d_groups, n_groups, d_cls, d_tab, d_slot_row, d_slot_nt, d_psi, d_scratch, rows, E, d_out, a_out,
             sample_base, step_begin, step_end, slice, mask_on, d_busy, d_progress, d_status, ring, wait_polls,
             nullptr, nullptr, 0);
-    } else if (d_ckpt) {
-        k_propagate_full_cn<false, true><<<(unsigned)ctas, P * kLanes, smem, st>>>(
+    } else {
+        auto kernel = d_ckpt ? (fix ? k_propagate_full_cn<false, true, true> : k_propagate_full_cn<false, true, false>)
+                             : (fix ? k_propagate_full_cn<false, false, true> : k_propagate_full_cn<false, false, false>);
+        kernel<<<(unsigned)ctas, P * kLanes, smem, st>>>(
             d_groups, n_groups, d_cls, d_tab, d_slot_row, d_slot_nt, d_psi, d_scratch, rows, E, d_out, a_out,
             sample_base, step_begin, step_end, slice, mask_on, d_busy, d_progress, d_status, ring, wait_polls,
             static_cast<double2*>(d_ckpt), d_ckpt_off, kc);
-    } else {
-        k_propagate_full_cn<false, false><<<(unsigned)ctas, P * kLanes, smem, st>>>(
-            d_groups, n_groups, d_cls, d_tab, d_slot_row, d_slot_nt, d_psi, d_scratch, rows, E, d_out, a_out,
-            sample_base, step_begin, step_end, slice, mask_on, d_busy, d_progress, d_status, ring, wait_polls,
-            nullptr, nullptr, 0);
     }
     return cudaGetLastError();
 }
 
 int propagate_ring_slots(int P, int per_sm) { return full_cn_ring_slots(P, per_sm); }
 
-int propagate_max_ctas_per_sm(int mixed, int P)
+int propagate_max_ctas_per_sm(int mixed, int fix, int P)
 {
     int n = 0;
-    const size_t smem = full_cn_smem_bytes(mixed, P, kMinRing);   // the shallowest ring
+    const size_t smem = full_cn_smem_bytes(mixed, fix, P, kMinRing);   // the shallowest ring
     if (mixed &&
-        cudaFuncSetAttribute(k_propagate_full_cn<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaFuncSetAttribute(k_propagate_full_cn<true, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)full_cn_smem_max_bytes()) != cudaSuccess) {
         cudaGetLastError();   // do not leave the failure for the next launch check
         return 1;
     }
-    const cudaError_t e = mixed ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_propagate_full_cn<true, false>, P * kLanes, smem)
-                                : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_propagate_full_cn<false, false>, P * kLanes, smem);
+    auto kernel = mixed ? k_propagate_full_cn<true, false, false>
+                        : (fix ? k_propagate_full_cn<false, false, true> : k_propagate_full_cn<false, false, false>);
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, P * kLanes, smem);
     if (e != cudaSuccess) return 1;
     return n > 0 ? n : 1;
 }

@@ -325,7 +325,7 @@ cudaError_t launch_broadcast_psi(int mixed, const GroupDesc* d_groups, int64_t n
 // polls before a MIXED bulk-copy wait gives up (the batch reports TDSE_ERR_TIMEOUT).  d_ckpt (FP64
 // only, NULL = none): the state after every kc-th step is also written to the adjoint's checkpoint
 // layout (group g at d_ckpt_off[g], checkpoint c at + c * N * I; c = 0 is the state at step 0).
-cudaError_t launch_propagate_full_cn(int mixed, const GroupDesc* d_groups, int64_t n_groups, int P, int ctas,
+cudaError_t launch_propagate_full_cn(int mixed, int fix, const GroupDesc* d_groups, int64_t n_groups, int P, int ctas,
                                      const ClassDesc* d_cls, const double* d_tab, const int64_t* d_slot_row,
                                      const int64_t* d_slot_nt, void* d_psi, void* d_scratch, int rows,
                                      const double* E, double* d_out, double* a_out, int64_t sample_base,
@@ -334,7 +334,7 @@ cudaError_t launch_propagate_full_cn(int mixed, const GroupDesc* d_groups, int64
                                      cudaStream_t st, void* d_ckpt = nullptr, const int64_t* d_ckpt_off = nullptr,
                                      int kc = 0);
 // CTAs of P warps that fit on one SM (MIXED: with the shallowest bulk-copy ring).
-int propagate_max_ctas_per_sm(int mixed, int P);
+int propagate_max_ctas_per_sm(int mixed, int fix, int P);
 // MIXED bulk-copy slots per warp when per_sm CTAs of P warps share an SM.
 int propagate_ring_slots(int P, int per_sm);
 
@@ -383,7 +383,7 @@ cudaError_t launch_resample_field(const double* coarse, int64_t n_rows, int M, d
                                   int64_t n_fine, int64_t out_stride, double* out, void* work, cudaStream_t st);
 
 // Persistent NUMEROV_SPLIT propagation (same scheduler, scratch and layouts; tables nw/nl/nc/nf).
-cudaError_t launch_propagate_numerov(int mixed, const GroupDesc* d_groups, int64_t n_groups, int P, int ctas,
+cudaError_t launch_propagate_numerov(int mixed, int fix, const GroupDesc* d_groups, int64_t n_groups, int P, int ctas,
                                      const ClassDesc* d_cls, const double* d_tab, const int64_t* d_slot_row,
                                      const int64_t* d_slot_nt, void* d_psi, void* d_scratch, int rows,
                                      const double* E, double* d_out, double* a_out, int64_t sample_base,
