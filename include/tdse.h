@@ -361,7 +361,8 @@ tdse_status tdse_model_layout(const tdse_instance* inst_host, int64_t n_inst, do
  * takes ctas x ckpt_every x warps x rows x 32 complex doubles (tdse_plan: ctas, warps_per_cta; rows
  * = segment + 2 halos); it is allocated at the next adjoint call when it takes at most half of the
  * device's free memory, and left out otherwise.  Results are bitwise the same with and without it.
- * Batches that the fixed-point adjoint serves (tdse_adjoint) neither allocate nor use it.
+ * Batches that the fixed-point adjoint serves (tdse_adjoint) allocate it for the groups that a call leaves to the
+ * FP64 sweeps.
  * enable: 1 (default) uses it when it fits, 0 never (and frees it).  The paper has no counterpart. */
 tdse_status tdse_set_adjoint_gamma_tape(tdse_batch* batch, int32_t enable);
 

@@ -102,3 +102,39 @@ def test_full_cn_fp64_sweeps(env, N, dx, dt, lanes):
         sl = slice(offs[i], offs[i + 1])
         assert _rel(d[sl].cpu().numpy(), d_o) < RTOL_SERIES and _rel(acc[sl].cpu().numpy(), a_o) < RTOL_SERIES, i
     b.close()
+
+
+@pytest.mark.parametrize("dx,dt,kc,field,lanes", [(0.2, 0.05, 37, 8.0, 1), (0.2, 0.05, 37, 8.0, 4), (0.1, 0.02, 37, 0.05, 1),
+                                                  (0.1, 0.02, 37, 0.05, 4), (0.2, 0.05, 400, 0.05, 1), (0.2, 0.05, 400, 0.05, 4)])
+def test_gamma_tape_of_the_fp64_adjoint(env, dx, dt, kc, field, lanes):
+    """The FP64 adjoint with and without its gamma tape gives the same bits, through both entry points: groups that
+    the fixed-point adjoint leaves (a field beyond the range), a class without that form, and an interval longer than
+    the grid.  Dropping the tape gives memory back, so it was there."""
+    tdse, oracle = env
+    rng = np.random.default_rng(kc)
+    n, N, a, nt = 35, 384, 1.19, 120
+    E = rng.uniform(-field, field, n * (nt + 1))
+    Et = torch.from_numpy(E).cuda()
+    gd, ga = (torch.from_numpy(rng.standard_normal(E.size)).cuda() for _ in range(2))
+    b = tdse.Batch([N] * n, dx, a, [nt] * n, dt, absorber=(10.0, 0.125), lanes_per_instance=lanes)
+    b.ground_state(**GS_KW)
+    psi0 = b.save_state()
+    d, acc = torch.zeros_like(Et), torch.zeros_like(Et)
+    out, free = [], []
+    for tape in (True, False):
+        b.set_adjoint_gamma_tape(tape)
+        b.load_state(psi0)
+        one = b.adjoint(Et, gd, ga, ckpt_every=kc)
+        b.propagate_checkpointed(Et, d, acc, kc)
+        out.append((one, b.adjoint_checkpointed(Et, gd, ga)))
+        torch.cuda.synchronize()
+        free.append(torch.cuda.mem_get_info()[0])
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+    assert free[1] - free[0] >= (4 << 20), free
+    p, m = oracle.ground_state(N, dx, a, **GS_KW)[0], oracle.mask(N, dx, 10.0, 0.125)
+    for i in (0, 17, n - 1):
+        sl = slice(i * (nt + 1), (i + 1) * (nt + 1))
+        ref = oracle.adjoint(p, E[sl], dx, dt, a, gd[sl].cpu().numpy(), ga[sl].cpu().numpy(), mask_values=m)
+        for g in out[0]:
+            assert _rel(g[sl].cpu().numpy(), ref) < RTOL_SERIES, i
+    b.close()
