@@ -246,7 +246,8 @@ tdse_status tdse_populations(tdse_batch* batch, double r_core, double* out_dev, 
  * samples exactly.  It is T-periodic: times beyond the window wrap around, so pad the coarse row
  * with zeros past the pulse.  With out_stride equal to a batch's row stride the output feeds
  * tdse_propagate directly.  M in [2, 8192]; computed in FP64; synchronous (allocates coefficients and
- * transform nodes for a bounded number of rows and 132 bytes per output sample for the call). */
+ * transform nodes for a bounded number of rows and 132 bytes per output sample of a bounded number of these, less
+ * where the device has no room for that). */
 tdse_status tdse_resample_field(const double* coarse_dev, int64_t n_rows, int32_t M, double dt_coarse, double dt_fine,
                                 int64_t n_fine, int64_t out_stride, double* out_dev, int device, void* stream);
 

@@ -1331,10 +1331,19 @@ tdse_status tdse_resample_field(const double* coarse_dev, int64_t n_rows, int32_
     DeviceGuard guard(device);
     if (!guard.ok) return fail(TDSE_ERR_CUDA, "cudaSetDevice failed");
     cudaStream_t st = (cudaStream_t)stream;
+    // passes of up to 512 MB of rows and 128 MB of outputs, smaller ones where the device has no room for these
     void* d_work = nullptr;
-    cudaError_t e = cudaMallocAsync(&d_work, resample_field_bytes(resample_field_rows(n_rows, M), M, n_fine), st);
+    size_t room = size_t(512) << 20;
+    FieldPlan plan = resample_field_plan(n_rows, M, n_fine, room);
+    cudaError_t e = cudaMallocAsync(&d_work, plan.bytes, st);
+    while (e == cudaErrorMemoryAllocation && room > (size_t(1) << 20)) {
+        cudaGetLastError();
+        room /= 8;
+        plan = resample_field_plan(n_rows, M, n_fine, room);
+        e = cudaMallocAsync(&d_work, plan.bytes, st);
+    }
     if (e == cudaSuccess) {
-        e = launch_resample_field(coarse_dev, n_rows, M, dt_coarse, dt_fine, n_fine, out_stride, out_dev, d_work, st);
+        e = launch_resample_field(coarse_dev, n_rows, M, dt_coarse, dt_fine, n_fine, out_stride, out_dev, plan, d_work, st);
         const cudaError_t f = cudaFreeAsync(d_work, st);
         if (e == cudaSuccess) e = f;
     }

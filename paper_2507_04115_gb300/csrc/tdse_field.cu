@@ -31,6 +31,7 @@ namespace tdse {
 namespace {
 
 constexpr int kWin = 16;            // nodes under the window
+static_assert(kWin * sizeof(double) + sizeof(int) == kFieldOutputBytes, "tables per output");
 constexpr int kInterpRows = 8;      // rows per thread of the interpolation
 constexpr int kGridThreads = 512;
 constexpr double kPi = 3.14159265358979323846;
@@ -50,8 +51,18 @@ __device__ double bessel_i0(double x, const double* r)
     return s;
 }
 
-__global__ void k_field_tables(int M, int G, double b, double dt_f, double T, int64_t n_fine, double2* __restrict__ tw_m,
-                               double2* __restrict__ tw_g, int* __restrict__ node, double* __restrict__ wgt)
+// n dt_f / T as a pair of doubles
+__device__ __forceinline__ void periods(int64_t n, double dt_f, double T, double& q, double& ql)
+{
+    const double t = (double)n * dt_f, tl = fma((double)n, dt_f, -t);
+    q = t / T;
+    ql = (fma(-q, T, t) + tl) / T;
+}
+
+// The tables of outputs n_first .. n_first + n_cnt - 1.
+__global__ void k_field_tables(int M, int G, double b, double dt_f, double T, int64_t n_first, int64_t n_cnt,
+                               double2* __restrict__ tw_m, double2* __restrict__ tw_g, int* __restrict__ node,
+                               double* __restrict__ wgt)
 {
     __shared__ double inv_k2[kI0Terms];
     for (int k = threadIdx.x; k < kI0Terms; k += blockDim.x) inv_k2[k] = k > 0 ? 1.0 / ((double)k * k) : 0.0;
@@ -67,17 +78,17 @@ __global__ void k_field_tables(int M, int G, double b, double dt_f, double T, in
         sincospi(2.0 * (double)i / (double)G, &s, &c);
         tw_g[i] = make_double2(c, s);
     }
-    if (i < n_fine * kWin) {
+    if (i < n_cnt * kWin) {
         const int64_t n = i / kWin;
         const int j = (int)(i % kWin);
-        // x = G frac(n dt_f / T) as a node number and a remainder, the quotient in a pair of doubles
-        const double t = (double)n * dt_f, tl = fma((double)n, dt_f, -t);
-        const double q = t / T, ql = (fma(-q, T, t) + tl) / T;
+        // x = G frac(n dt_f / T) as a node number and a remainder
+        double q, ql;
+        periods(n_first + n, dt_f, T, q, ql);
         const double xh = (q - floor(q)) * G, l = floor(xh);
         const double z = (xh - l) + ql * G;            // offset from node l, in [0, 1] to rounding
         const double y = (z + (kWin / 2 - 1) - j) * (2.0 / kWin);
         const double r = 1.0 - y * y;
-        wgt[j * n_fine + n] = r > 0.0 ? bessel_i0(b * sqrt(r), inv_k2) : 0.0;   // phi up to the factor in k_field_grid
+        wgt[j * n_cnt + n] = r > 0.0 ? bessel_i0(b * sqrt(r), inv_k2) : 0.0;   // phi up to the factor in k_field_grid
         if (j == 0) node[n] = ((int)l - (kWin / 2 - 1) + G) & (G - 1);
     }
 }
@@ -165,15 +176,16 @@ k_field_grid(const double2* __restrict__ coef, int K, int G, int log_n, const do
     for (int n = threadIdx.x; n < N; n += blockDim.x) g[n] = z[n];
 }
 
+// Outputs n_first .. n_first + n_cnt - 1 of the rows (out at output n_first).
 __global__ void __launch_bounds__(256)
-k_field_interp(const double* __restrict__ grid, int64_t n_rows, int G, int64_t n_fine, int64_t out_stride,
+k_field_interp(const double* __restrict__ grid, int64_t n_rows, int G, int64_t n_cnt, int64_t out_stride,
                const int* __restrict__ node, const double* __restrict__ wgt, double* __restrict__ out)
 {
     const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= n_fine) return;
+    if (n >= n_cnt) return;
     double w[kWin];
 #pragma unroll
-    for (int j = 0; j < kWin; ++j) w[j] = wgt[j * n_fine + n];
+    for (int j = 0; j < kWin; ++j) w[j] = wgt[j * n_cnt + n];
     const int l0 = node[n];
     const int64_t r0 = (int64_t)blockIdx.y * kInterpRows, r1 = min(n_rows, r0 + kInterpRows);
     for (int64_t r = r0; r < r1; ++r) {
@@ -190,34 +202,12 @@ k_field_interp(const double* __restrict__ grid, int64_t n_rows, int G, int64_t n
 
 }  // namespace
 
-// Nodes of the oversampled grid: at least 4 per highest harmonic, and room for the window.
-static int field_nodes(int M)
-{
-    int G = 64;
-    while (G < 4 * (M / 2)) G *= 2;
-    return G;
-}
-
-size_t resample_field_bytes(int64_t rows, int M, int64_t n_fine)
-{
-    const int G = field_nodes(M);
-    return sizeof(double2) * ((size_t)M + G / 2) + sizeof(double) * (size_t)kWin * n_fine + ((sizeof(int) * (size_t)n_fine + 15) & ~size_t(15)) +
-           (size_t)rows * (sizeof(double2) * (M / 2 + 1) + sizeof(double) * G);
-}
-
-// rows per pass: their grids and coefficients below 512 MB
-int64_t resample_field_rows(int64_t n_rows, int M)
-{
-    const int64_t per = (int64_t)sizeof(double2) * (M / 2 + 1) + (int64_t)sizeof(double) * field_nodes(M);
-    return std::max<int64_t>(1, std::min<int64_t>({n_rows, (int64_t(512) << 20) / per, 65535}));
-}
-
 cudaError_t launch_resample_field(const double* coarse, int64_t n_rows, int M, double dt_c, double dt_f,
-                                  int64_t n_fine, int64_t out_stride, double* out, void* work, cudaStream_t st)
+                                  int64_t n_fine, int64_t out_stride, double* out, const FieldPlan& plan, void* work,
+                                  cudaStream_t st)
 {
     if (n_rows == 0 || n_fine == 0) return cudaSuccess;
     const int K = M / 2, G = field_nodes(M);
-    const int64_t chunk = resample_field_rows(n_rows, M);
     static std::atomic<bool> attr_set[kMaxAttrDevices];   // rows up to 8192 samples: 64 and 128 KB of shared memory
     int dev = 0;
     if (attr_needed(attr_set, &dev)) {
@@ -230,22 +220,30 @@ cudaError_t launch_resample_field(const double* coarse, int64_t n_rows, int M, d
     double2* tw_m = static_cast<double2*>(work);
     double2* tw_g = tw_m + M;
     double2* coef = tw_g + G / 2;
-    double* grid = reinterpret_cast<double*>(coef + chunk * (K + 1));
-    double* wgt = grid + chunk * G;
-    int* node = reinterpret_cast<int*>(wgt + kWin * n_fine);
-    const double b = kPi * kWin * (1.0 - (double)K / G);
+    double* grid = reinterpret_cast<double*>(coef + plan.rows * (K + 1));
+    double* wgt = grid + plan.rows * G;
+    int* node = reinterpret_cast<int*>(wgt + kWin * plan.outputs);
+    const double T = M * dt_c, b = kPi * kWin * (1.0 - (double)K / G);
     int log_n = 0;
     while ((1 << log_n) < G / 2) ++log_n;
-    const int64_t items = std::max<int64_t>({(int64_t)M, (int64_t)G / 2, n_fine * kWin});
-    k_field_tables<<<(unsigned)((items + 255) / 256), 256, 0, st>>>(M, G, b, dt_f, M * dt_c, n_fine, tw_m, tw_g, node, wgt);
+    auto tables = [&](int64_t n0, int64_t cnt) {
+        const int64_t items = std::max<int64_t>({(int64_t)M, (int64_t)G / 2, cnt * kWin});
+        k_field_tables<<<(unsigned)((items + 255) / 256), 256, 0, st>>>(M, G, b, dt_f, T, n0, cnt, tw_m, tw_g, node, wgt);
+    };
+    const bool one = plan.outputs >= n_fine;   // every output's window fits: built once for all rows
+    tables(0, one ? n_fine : 0);
     cudaError_t e = cudaGetLastError();
-    for (int64_t r0 = 0; e == cudaSuccess && r0 < n_rows; r0 += chunk) {
-        const int64_t nr = std::min(chunk, n_rows - r0);
+    for (int64_t r0 = 0; e == cudaSuccess && r0 < n_rows; r0 += plan.rows) {
+        const int64_t nr = std::min(plan.rows, n_rows - r0);
         k_field_coeffs<<<dim3((unsigned)((K + 128) / 128), (unsigned)nr), 128, sizeof(double) * 2 * ((M - 1) / 2 + 1), st>>>(
             coarse + r0 * M, M, G, b, tw_m, coef);
         k_field_grid<<<(unsigned)nr, kGridThreads, sizeof(double2) * (G / 2), st>>>(coef, K, G, log_n, tw_g, grid);
-        k_field_interp<<<dim3((unsigned)((n_fine + 255) / 256), (unsigned)((nr + kInterpRows - 1) / kInterpRows)), 256, 0, st>>>(
-            grid, nr, G, n_fine, out_stride, node, wgt, out + r0 * out_stride);
+        for (int64_t n0 = 0; n0 < n_fine; n0 += plan.outputs) {
+            const int64_t cnt = std::min(plan.outputs, n_fine - n0);
+            if (!one) tables(n0, cnt);
+            k_field_interp<<<dim3((unsigned)((cnt + 255) / 256), (unsigned)((nr + kInterpRows - 1) / kInterpRows)), 256, 0, st>>>(
+                grid, nr, G, cnt, out_stride, node, wgt, out + r0 * out_stride + n0);
+        }
         e = cudaGetLastError();
     }
     return e;

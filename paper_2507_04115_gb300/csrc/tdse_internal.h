@@ -11,6 +11,7 @@
 
 #include "tdse.h"
 #include "tdse_fix.cuh"
+#include "tdse_rules.h"
 
 namespace tdse {
 
@@ -376,11 +377,10 @@ cudaError_t launch_ionisation(const double* d_P, int64_t n_inst, int nE, const d
                               int sm_count, cudaStream_t st);
 
 // Field ingestion (tdse_field.cu): the zero-padded interpolant of every coarse row at n_fine samples.
-// work: resample_field_bytes(resample_field_rows(n_rows, M), M, n_fine) bytes.
-size_t resample_field_bytes(int64_t rows, int M, int64_t n_fine);
-int64_t resample_field_rows(int64_t n_rows, int M);
+// work: plan.bytes.
 cudaError_t launch_resample_field(const double* coarse, int64_t n_rows, int M, double dt_c, double dt_f,
-                                  int64_t n_fine, int64_t out_stride, double* out, void* work, cudaStream_t st);
+                                  int64_t n_fine, int64_t out_stride, double* out, const FieldPlan& plan, void* work,
+                                  cudaStream_t st);
 
 // Persistent NUMEROV_SPLIT propagation (same scheduler, scratch and layouts; tables nw/nl/nc/nf).
 cudaError_t launch_propagate_numerov(int mixed, int fix, const GroupDesc* d_groups, int64_t n_groups, int P, int ctas,

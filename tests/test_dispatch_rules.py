@@ -1,0 +1,39 @@
+"""The host rules of the batch-free entry points (csrc/tdse_rules.h), compiled for the host."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2507_04115_gb300", "csrc")
+
+
+def _run(tmp_path, body):
+    if shutil.which("g++") is None:
+        pytest.skip("g++ not found")
+    src, exe = tmp_path / "t.cpp", tmp_path / "t"
+    src.write_text('#include "tdse_rules.h"\n#include <cstdio>\nusing namespace tdse;\nint main() {\n%s\nreturn 0; }\n' % body)
+    subprocess.run(["g++", "-std=c++17", "-I" + CSRC, "-o", str(exe), str(src)], check=True)
+    r = subprocess.run([str(exe)], capture_output=True, text=True)
+    assert r.returncode == 0, (r.returncode, r.stdout)
+
+
+def test_field_passes_are_bounded(tmp_path):
+    """The scratch of a resampling pass stays within 5/4 of its room and the twiddles, however many rows and outputs
+    there are, down to a pass of one row and one output."""
+    _run(tmp_path, """
+    const size_t MB = size_t(1) << 20;
+    for (size_t room = 512 * MB; room >= MB / 2; room /= 8)
+        for (int M : {2, 3, 100, 2400, 8191, 8192})
+            for (int64_t rows : {int64_t(1), int64_t(7), int64_t(100000), int64_t(1) << 31})
+                for (int64_t n : {int64_t(1), int64_t(55160), int64_t(1000000000), int64_t(1) << 40}) {
+                    const FieldPlan p = resample_field_plan(rows, M, n, room);
+                    if (p.rows < 1 || p.rows > rows || p.rows > 65535 || p.outputs < 1 || p.outputs > n) return 1;
+                    const size_t least = 16 * (size_t)(M / 2 + 1) + 8 * (size_t)field_nodes(M) + 132;   // one row, one output
+                    const size_t twiddles = 16 * (size_t)(M + field_nodes(M) / 2);
+                    if (p.bytes > room + room / 4 + least + twiddles) return 2;
+                    if (p.bytes < (size_t)p.rows * 8 * field_nodes(M) + (size_t)p.outputs * 132 + twiddles) return 3;
+                }
+    const FieldPlan p = resample_field_plan(256, 2400, 55160, 512 * MB);   // a workload's call: one pass
+    if (p.rows != 256 || p.outputs != 55160) return 4;
+    """)
