@@ -1335,19 +1335,23 @@ tdse_status tdse_resample_field(const double* coarse_dev, int64_t n_rows, int32_
     void* d_work = nullptr;
     size_t room = size_t(512) << 20;
     FieldPlan plan = resample_field_plan(n_rows, M, n_fine, room);
-    cudaError_t e = cudaMallocAsync(&d_work, plan.bytes, st);
+    // (the direct sum's few kilobytes come from the ordinary heap: the pool, trimmed at every synchronisation, costs a small
+    // call 20 us)
+    auto take = [&]() { return plan.direct ? cudaMalloc(&d_work, plan.bytes) : cudaMallocAsync(&d_work, plan.bytes, st); };
+    cudaError_t e = take();
     while (e == cudaErrorMemoryAllocation && room > (size_t(1) << 20)) {
         cudaGetLastError();
         room /= 8;
         plan = resample_field_plan(n_rows, M, n_fine, room);
-        e = cudaMallocAsync(&d_work, plan.bytes, st);
+        e = take();
     }
     if (e == cudaSuccess) {
         e = launch_resample_field(coarse_dev, n_rows, M, dt_coarse, dt_fine, n_fine, out_stride, out_dev, plan, d_work, st);
-        const cudaError_t f = cudaFreeAsync(d_work, st);
+        const cudaError_t f = plan.direct ? cudaSuccess : cudaFreeAsync(d_work, st);
         if (e == cudaSuccess) e = f;
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (plan.direct && d_work) cudaFree(d_work);
     if (e != cudaSuccess) return cuda_fail(e, "tdse_resample_field");
     return TDSE_OK;
 }

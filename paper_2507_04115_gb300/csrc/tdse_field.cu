@@ -20,6 +20,7 @@
 //                   difference the sine): M FP64 multiply-adds per coefficient, twiddles from a table
 //   k_field_grid    one CTA per row: the G node values by a complex FFT of length G / 2 in shared memory
 //   k_field_interp  16 multiply-adds per output
+//   k_field_direct  the sum over k itself, for few coefficients and rows (resample_field_plan)
 // Work per row: O(M^2 / 2 + G log G + 16 n_fine) FP64 instructions instead of O(3 M^2 + 3 M n_fine) for the
 // direct sums with turning twiddles.  Measured, 256 rows of 2400 samples to 55160: 217 ms by the direct
 // sums, 2.9 ms here: coefficients 1.8, tables 0.4, interpolation 0.4, grid 0.15.
@@ -93,7 +94,9 @@ __global__ void k_field_tables(int M, int G, double b, double dt_f, double T, in
     }
 }
 
-// c_k / phihat_k of every row, k = 0 .. K (one thread per k; the row's sums and differences in shared memory)
+// c_k / phihat_k of every row, k = 0 .. K (one thread per k; the row's sums and differences in shared memory); kDirect: c_k,
+// with twiddles of the block's own (one launch less for small calls)
+template <bool kDirect>
 __global__ void __launch_bounds__(128)
 k_field_coeffs(const double* __restrict__ coarse, int M, int G, double b, const double2* __restrict__ tw, double2* __restrict__ coef)
 {
@@ -106,6 +109,14 @@ k_field_coeffs(const double* __restrict__ coarse, int M, int G, double b, const 
         row[m] = x[m] + x[M - m];
         dif[m] = x[m] - x[M - m];
     }
+    double2* own = reinterpret_cast<double2*>(row + 2 * (H + 1));
+    if constexpr (kDirect)
+        for (int m = threadIdx.x; m < M; m += blockDim.x) {
+            double s, c;
+            sincospi(2.0 * (double)m / (double)M, &s, &c);
+            own[m] = make_double2(c, s);
+        }
+    auto twiddle = [&](int i) { return kDirect ? own[i] : __ldg(tw + i); };
     __syncthreads();
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k > K) return;
@@ -116,19 +127,21 @@ k_field_coeffs(const double* __restrict__ coarse, int M, int G, double b, const 
     double2 z = make_double2(0.0, 0.0);
     if (H > 0) {
         idx = k % M;
-        z = __ldg(tw + idx);
+        z = twiddle(idx);
     }
     for (int m = 1; m <= H; ++m) {
         const double2 c = z;
         idx += k;
         if (idx >= M) idx -= M;
-        z = __ldg(tw + idx);
+        z = twiddle(idx);
         sr = fma(row[m], c.x, sr);
         si = fma(-dif[m], c.y, si);
     }
-    // Kaiser-Bessel window's transform at xi = 2 pi k / G
-    const double xi = 2.0 * kPi * k / G, u = 0.5 * kWin * xi, v = sqrt(b * b - u * u);
-    const double f = (k == 0 || 2 * k == M ? 1.0 : 2.0) / M * v / (kWin * sinh(v));
+    double f = (k == 0 || 2 * k == M ? 1.0 : 2.0) / M;
+    if (!kDirect) {   // Kaiser-Bessel window's transform at xi = 2 pi k / G
+        const double xi = 2.0 * kPi * k / G, u = 0.5 * kWin * xi, v = sqrt(b * b - u * u);
+        f = f * v / (kWin * sinh(v));
+    }
     coef[r * (K + 1) + k] = make_double2(f * sr, f * si);
 }
 
@@ -176,6 +189,43 @@ k_field_grid(const double2* __restrict__ coef, int K, int G, int log_n, const do
     for (int n = threadIdx.x; n < N; n += blockDim.x) g[n] = z[n];
 }
 
+// The direct sum, an output per thread: Horner's rule in z = e^{2 pi i t / T} over blocks of 64 coefficients, each
+// block times z to its first index (from a sincospi of its own: an error of z counts at most 63 times).
+__global__ void __launch_bounds__(256)
+k_field_direct(const double2* __restrict__ coef, int K, double dt_f, double T, int64_t n_fine, int64_t out_stride,
+               double* __restrict__ out)
+{
+    extern __shared__ double2 c[];
+    const int64_t r = blockIdx.y;
+    for (int k = threadIdx.x; k <= K; k += blockDim.x) c[k] = coef[r * (K + 1) + k];
+    __syncthreads();
+    const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (n >= n_fine) return;
+    double q, ul;
+    periods(n, dt_f, T, q, ul);
+    const double uh = q - floor(q);
+    auto power = [&](int k) {   // z^k
+        const double ph = k * uh, pl = (fma((double)k, uh, -ph) + k * ul) * (2.0 * kPi);
+        double s, co;
+        sincospi(2.0 * (ph - floor(ph)), &s, &co);
+        return make_double2(fma(-pl, s, co), fma(pl, co, s));
+    };
+    const double2 z = power(1);
+    double sum = 0.0;
+    for (int k0 = 0; k0 <= K; k0 += 64) {
+        int k = min(k0 + 63, K);
+        double hr = c[k].x, hi = c[k].y;
+        for (--k; k >= k0; --k) {
+            const double t = fma(hr, z.x, fma(-hi, z.y, c[k].x));
+            hi = fma(hr, z.y, fma(hi, z.x, c[k].y));
+            hr = t;
+        }
+        const double2 p = power(k0);
+        sum = fma(hr, p.x, fma(-hi, p.y, sum));
+    }
+    out[r * out_stride + n] = sum;
+}
+
 // Outputs n_first .. n_first + n_cnt - 1 of the rows (out at output n_first).
 __global__ void __launch_bounds__(256)
 k_field_interp(const double* __restrict__ grid, int64_t n_rows, int G, int64_t n_cnt, int64_t out_stride,
@@ -207,23 +257,23 @@ cudaError_t launch_resample_field(const double* coarse, int64_t n_rows, int M, d
                                   cudaStream_t st)
 {
     if (n_rows == 0 || n_fine == 0) return cudaSuccess;
-    const int K = M / 2, G = field_nodes(M);
+    const int K = M / 2, G = plan.direct ? 0 : field_nodes(M);
     static std::atomic<bool> attr_set[kMaxAttrDevices];   // rows up to 8192 samples: 64 and 128 KB of shared memory
     int dev = 0;
     if (attr_needed(attr_set, &dev)) {
-        cudaError_t e = cudaFuncSetAttribute(k_field_coeffs, cudaFuncAttributeMaxDynamicSharedMemorySize, 8192 * 8);
+        cudaError_t e = cudaFuncSetAttribute(k_field_coeffs<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 8192 * 8);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_field_grid, cudaFuncAttributeMaxDynamicSharedMemorySize, 8192 * 16);
         if (e != cudaSuccess) return e;
         attr_done(attr_set, dev);
     }
     double2* tw_m = static_cast<double2*>(work);
-    double2* tw_g = tw_m + M;
+    double2* tw_g = tw_m + (plan.direct ? 0 : M);
     double2* coef = tw_g + G / 2;
     double* grid = reinterpret_cast<double*>(coef + plan.rows * (K + 1));
     double* wgt = grid + plan.rows * G;
     int* node = reinterpret_cast<int*>(wgt + kWin * plan.outputs);
-    const double T = M * dt_c, b = kPi * kWin * (1.0 - (double)K / G);
+    const double T = M * dt_c, b = plan.direct ? 0.0 : kPi * kWin * (1.0 - (double)K / G);
     int log_n = 0;
     while ((1 << log_n) < G / 2) ++log_n;
     auto tables = [&](int64_t n0, int64_t cnt) {
@@ -231,12 +281,20 @@ cudaError_t launch_resample_field(const double* coarse, int64_t n_rows, int M, d
         k_field_tables<<<(unsigned)((items + 255) / 256), 256, 0, st>>>(M, G, b, dt_f, T, n0, cnt, tw_m, tw_g, node, wgt);
     };
     const bool one = plan.outputs >= n_fine;   // every output's window fits: built once for all rows
-    tables(0, one ? n_fine : 0);
+    if (!plan.direct) tables(0, one ? n_fine : 0);
     cudaError_t e = cudaGetLastError();
     for (int64_t r0 = 0; e == cudaSuccess && r0 < n_rows; r0 += plan.rows) {
         const int64_t nr = std::min(plan.rows, n_rows - r0);
-        k_field_coeffs<<<dim3((unsigned)((K + 128) / 128), (unsigned)nr), 128, sizeof(double) * 2 * ((M - 1) / 2 + 1), st>>>(
-            coarse + r0 * M, M, G, b, tw_m, coef);
+        const dim3 cgrid((unsigned)((K + 128) / 128), (unsigned)nr);
+        const size_t csmem = sizeof(double) * 2 * ((M - 1) / 2 + 1);
+        if (plan.direct) {
+            k_field_coeffs<true><<<cgrid, 128, csmem + sizeof(double2) * M, st>>>(coarse + r0 * M, M, G, b, nullptr, coef);
+            k_field_direct<<<dim3((unsigned)((n_fine + 255) / 256), (unsigned)nr), 256, sizeof(double2) * (K + 1), st>>>(
+                coef, K, dt_f, T, n_fine, out_stride, out + r0 * out_stride);
+            e = cudaGetLastError();
+            continue;
+        }
+        k_field_coeffs<false><<<cgrid, 128, csmem, st>>>(coarse + r0 * M, M, G, b, tw_m, coef);
         k_field_grid<<<(unsigned)nr, kGridThreads, sizeof(double2) * (G / 2), st>>>(coef, K, G, log_n, tw_g, grid);
         for (int64_t n0 = 0; n0 < n_fine; n0 += plan.outputs) {
             const int64_t cnt = std::min(plan.outputs, n_fine - n0);

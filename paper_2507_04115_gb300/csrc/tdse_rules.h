@@ -21,20 +21,35 @@ inline int field_nodes(int M)
 // Bytes of the tables of an output (16 weights and a node).
 constexpr int64_t kFieldOutputBytes = 132;
 
+// Is the sum over k the quicker way?  In us: it takes rows x (3 M + 84) FP64 instructions per output (4 per coefficient and
+// the phases) behind a chain of M / 2 coefficients; the grid takes 4700 per output for the window's weights, whatever the
+// rows, 16 more per row, and the chains of its passes.  Measured, whole calls, direct and by the grid: 1 row of 100
+// samples to 400000 outputs 416 and 2880 us, 8 of 100 to 55160 462 and 605, 16 of 100 683 and 620, 4 of 300 to 12000
+// 327 and 342, 1 of 600 to 1000 329 and 286, 1 of 1200 to 400000 2256 and 3067, 2 of them 4023 and 3083.
+inline bool field_direct(int64_t n_rows, int M, int64_t n_fine)
+{
+    const double r = (double)n_rows, n = (double)n_fine;
+    const double direct = 0.17 * M + 1.4e-6 * n * r * (3.0 * M + 84.0);
+    const double grid = 25.0 + 0.085 * M + 1.4e-6 * n * (4700.0 + 16.0 * r);
+    return M <= 2000 && direct < grid;   // (M: samples and twiddles fit 48 KB of shared memory)
+}
+
 // Rows and outputs of a pass: the rows' coefficients and grids take at most `room` bytes, the outputs' tables a quarter
 // of it (or those of one row, of one output).  bytes: the scratch of such a pass.
 struct FieldPlan {
+    bool direct;   // the sum over k itself: no grid, no tables per output
     int64_t rows, outputs;
     size_t bytes;
 };
 inline FieldPlan resample_field_plan(int64_t n_rows, int M, int64_t n_fine, size_t room)
 {
-    const int G = field_nodes(M);
-    const int64_t per_row = 16 * (int64_t)(M / 2 + 1) + 8 * (int64_t)G;
     FieldPlan p;
+    p.direct = field_direct(n_rows, M, n_fine);
+    const int G = p.direct ? 0 : field_nodes(M);
+    const int64_t per_row = 16 * (int64_t)(M / 2 + 1) + 8 * (int64_t)G;
     p.rows = std::max<int64_t>(1, std::min<int64_t>({n_rows, (int64_t)room / per_row, 65535}));
-    p.outputs = std::max<int64_t>(1, std::min<int64_t>(n_fine, (int64_t)(room / 4) / kFieldOutputBytes));
-    p.bytes = 16 * ((size_t)M + G / 2) + (size_t)p.rows * per_row + (size_t)p.outputs * kFieldOutputBytes;
+    p.outputs = p.direct ? 0 : std::max<int64_t>(1, std::min<int64_t>(n_fine, (int64_t)(room / 4) / kFieldOutputBytes));
+    p.bytes = (p.direct ? 0 : 16 * ((size_t)M + G / 2)) + (size_t)p.rows * per_row + (size_t)p.outputs * kFieldOutputBytes;
     return p;
 }
 

@@ -28,12 +28,26 @@ def test_field_passes_are_bounded(tmp_path):
             for (int64_t rows : {int64_t(1), int64_t(7), int64_t(100000), int64_t(1) << 31})
                 for (int64_t n : {int64_t(1), int64_t(55160), int64_t(1000000000), int64_t(1) << 40}) {
                     const FieldPlan p = resample_field_plan(rows, M, n, room);
-                    if (p.rows < 1 || p.rows > rows || p.rows > 65535 || p.outputs < 1 || p.outputs > n) return 1;
+                    if (p.rows < 1 || p.rows > rows || p.rows > 65535 || p.outputs < (p.direct ? 0 : 1) || p.outputs > n) return 1;
                     const size_t least = 16 * (size_t)(M / 2 + 1) + 8 * (size_t)field_nodes(M) + 132;   // one row, one output
                     const size_t twiddles = 16 * (size_t)(M + field_nodes(M) / 2);
                     if (p.bytes > room + room / 4 + least + twiddles) return 2;
-                    if (p.bytes < (size_t)p.rows * 8 * field_nodes(M) + (size_t)p.outputs * 132 + twiddles) return 3;
+                    if (!p.direct && p.bytes < (size_t)p.rows * 8 * field_nodes(M) + (size_t)p.outputs * 132 + twiddles) return 3;
+                    if (p.direct && p.bytes < (size_t)p.rows * 16 * (M / 2 + 1)) return 3;
                 }
     const FieldPlan p = resample_field_plan(256, 2400, 55160, 512 * MB);   // a workload's call: one pass
     if (p.rows != 256 || p.outputs != 55160) return 4;
+    """)
+
+
+def test_field_route_follows_the_measured_calls(tmp_path):
+    """(rows, M, outputs) measured at least 10 % apart: the quicker route."""
+    _run(tmp_path, """
+    struct { int64_t rows; int M; int64_t n; bool direct; } c[] = {
+        {1, 2, 1000, true}, {32, 2, 1000, true}, {1, 600, 1000, false}, {1, 2400, 1000, false}, {1, 300, 12000, true},
+        {32, 100, 12000, false}, {4, 600, 12000, false}, {8, 100, 55160, true}, {16, 100, 55160, false}, {8, 300, 55160, false},
+        {1, 100, 400000, true}, {8, 100, 400000, true}, {32, 30, 400000, false}, {1, 1200, 400000, true}, {2, 1200, 400000, false},
+        {1, 2400, 55160, false}, {256, 2400, 55160, false}, {1, 8192, 1000000, false}};
+    for (auto& k : c)
+        if (field_direct(k.rows, k.M, k.n) != k.direct) { printf("%d %d\\n", (int)k.rows, k.M); return 1; }
     """)
