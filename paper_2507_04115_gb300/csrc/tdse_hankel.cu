@@ -18,9 +18,10 @@
 // (frequency, 128 observation radii); T is staged in shared memory by z' tiles (all threads read the
 // same element: broadcast), each thread owns one observation radius and sums over the tile.
 //   J0 comes from a table of its Taylor coefficients at the nodes x_i = i / 4 (k_j0_table, filled per call up
-// to the largest argument): |x - x_i| <= 1/8 and |J0^(n)| <= 1, so 12 terms leave (1/8)^12 / 12! < 4e-20.  A term
-// then costs 17 FP64 instructions (argument, node, 11 of the polynomial, 2 sums); CUDA's j0 took about
-// 200.  Measured, 32 x 32 points, 340 frequencies, 256 radii: 30 ms with j0, 3 ms with the table.
+// to the largest argument, where j0_table_nodes finds that it pays): |x - x_i| <= 1/8 and |J0^(n)| <= 1, so 12 terms
+// leave (1/8)^12 / 12! < 4e-20.  A term then costs 17 FP64 instructions (argument, node, 11 of the polynomial, 2 sums);
+// CUDA's j0 takes about 120 beyond x = 8.  Measured, 32 x 32 points, 340 frequencies, 256 radii: 7.1 ms with j0 and
+// 3.4 with the table at arguments up to 20, 14.9 and 3.7 up to 500.
 #include "tdse.h"
 #include "tdse_internal.h"
 
@@ -77,7 +78,6 @@ __global__ void k_dipole_spectrum(const double* __restrict__ a, const int64_t* _
 }
 
 constexpr int kJ0Terms = 12;
-constexpr int kJ0MaxNodes = 16384;   // 1.5 MB of coefficients, arguments up to 4096
 
 // Taylor coefficients J0^(n)(x_i) / n!, n < 12, at x_i = i / 4, layout [n][node], from
 //     J0^(n) = 2^-n sum_k (-1)^k C(n, k) J_{2k-n},  J_{-m} = (-1)^m J_m,
@@ -316,12 +316,19 @@ extern "C" tdse_status tdse_hankel(const double* S_dev, const double* rho_src_ho
     // nodes of the J0 table up to the largest argument k rho_o rho' / D
     const double x_max = *std::max_element(k_host, k_host + n_omega) * *std::max_element(rho_obs_host, rho_obs_host + n_obs) *
                          rho_src_host[n_rho - 1] / (z_obs - z_src_host[n_z - 1]);
-    const int nodes = (int)std::min(4.0 * x_max + 3.0, (double)kJ0MaxNodes);
+    int sms = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+    int nodes = j0_table_nodes(x_max, n_rho, n_z, n_omega, n_obs, sms);
     double* d_g = nullptr;
     cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&d_g), sizeof(double) * (g.size() + (size_t)kJ0Terms * nodes), st);
+    if (e == cudaErrorMemoryAllocation && nodes > 0) {   // no room for the table: j0
+        cudaGetLastError();
+        nodes = 0;
+        e = cudaMallocAsync(reinterpret_cast<void**>(&d_g), sizeof(double) * g.size(), st);
+    }
     if (e == cudaSuccess) e = cudaMemcpyAsync(d_g, g.data(), sizeof(double) * g.size(), cudaMemcpyHostToDevice, st);
     double* d_tab = d_g ? d_g + g.size() : nullptr;
-    if (e == cudaSuccess) {
+    if (e == cudaSuccess && nodes > 0) {
         k_j0_table<<<(nodes + 63) / 64, 64, 0, st>>>(nodes, d_tab);
         e = cudaGetLastError();
     }
