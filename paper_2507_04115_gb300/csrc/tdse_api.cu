@@ -1374,9 +1374,11 @@ tdse_status tdse_spectrum(const double* a_dev, const int64_t* offsets_host, int6
         shortest = std::min(shortest, L);
         longest = std::max(longest, L);
     }
-    int B = 0, P = 0;
+    int B = 0, P = 0, dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (shortest > 0 && longest < (int64_t(1) << 30) && 2 * (k_end - 1) < shortest && band_dft_allowed(st) &&
-        dft_plan(shortest, 2.0 * 3.14159265358979323846 * (double)(k_end - 1) / (double)shortest, k_end - k_begin, &B, &P)) {
+        dft_plan(shortest, 2.0 * 3.14159265358979323846 * (double)(k_end - 1) / (double)shortest, k_end - k_begin, n_rows, sms,
+                 &B, &P)) {
         const cudaError_t eb = launch_band_dft(a_dev, offsets_host, n_rows, dt, nullptr, k_begin, k_end - k_begin, B, P, nullptr, S_dev, st);
         if (eb == cudaSuccess) return TDSE_OK;
         if (eb != cudaErrorMemoryAllocation) return cuda_fail(eb, "tdse_spectrum");

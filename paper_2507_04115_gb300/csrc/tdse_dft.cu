@@ -17,10 +17,10 @@
 // recurrence in pairs of doubles; the block phases from products in pairs of doubles (or, for the bins,
 // from k (2 c_b) mod 2 L in integers), re-seeded every 16 blocks.
 //
-// B and P come from dft_plan, which minimises the instruction count L (P/2 + 1) + n_w (L / B)(P + 6) over
-// them.  Measured, 512 rows of 55160 samples, 400 bins: 170 ms by the direct sum, 4.1 ms here (B = 512,
+// B and P come from dft_plan (tdse_rules.h), which minimises the instruction count L (P/2 + 1) + n_w (L / B)(P + 6)
+// over them.  Measured, 512 rows of 55160 samples, 400 bins: 170 ms by the direct sum, 4.1 ms here (B = 512,
 // P = 40); both kernels are bound by the FP64 pipe.  The direct sum stays where the band is too wide for
-// blocks or has too few frequencies, on a capturing stream, and without room for the moments.
+// blocks or has too few frequencies, for short rows (dft_plan), on a capturing stream, and without room for the moments.
 #include "tdse_internal.h"
 
 #include <algorithm>
@@ -283,28 +283,6 @@ cudaError_t run_band(const double* a, const int64_t* d_offs, const int64_t* d_bo
 }
 
 }  // namespace
-
-bool dft_plan(int64_t samples, double turn, int64_t n_w, int* B_out, int* P_out)
-{
-    if (n_w < 32 || samples < 256 || !(turn < 0.8)) return false;
-    double best = 0.5 * 6.0 * (double)n_w;   // the direct sum per sample; the blocks have to halve it
-    int best_B = 0, best_P = 0;
-    for (int B = 32; B <= 1024; B *= 2)
-        for (int P = 16; P <= 40; P += 8) {
-            const double phi = 0.5 * turn * B;
-            if (phi > 0.0 && P * std::log(0.5 * phi) - std::lgamma(P + 1.0) + std::log(2.0) > std::log(1e-17)) continue;
-            const double cost = 0.5 * P + 1.0 + (double)n_w * (P + 6.0) / B;
-            if (cost < best) {
-                best = cost;
-                best_B = B;
-                best_P = P;
-            }
-            break;
-        }
-    *B_out = best_B;
-    *P_out = best_P;
-    return best_B > 0;
-}
 
 bool band_dft_allowed(cudaStream_t st)
 {

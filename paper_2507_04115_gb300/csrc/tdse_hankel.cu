@@ -249,8 +249,9 @@ extern "C" tdse_status tdse_dipole_spectrum(const double* a_dev, const int64_t* 
     for (int w = 0; w < n_omega; ++w) turn = std::max(turn, std::fabs(omega_host[w]) * dt);
     int64_t longest = 0;
     for (int64_t r = 0; r < n_rows; ++r) longest = std::max(longest, offsets_host[r + 1] - offsets_host[r]);
-    int B = 0, P = 0;
-    if (band_dft_allowed(st) && dft_plan(longest, turn, n_omega, &B, &P)) {   // frequencies far below the sampling rate: by block moments
+    int B = 0, P = 0, dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (band_dft_allowed(st) && dft_plan(longest, turn, n_omega, n_rows, sms, &B, &P)) {   // frequencies far below the sampling rate: by block moments
         const cudaError_t eb = launch_band_dft(a_dev, offsets_host, n_rows, dt, omega_host, 0, n_omega, B, P, weight_dev, out_dev, st);
         if (eb == cudaSuccess) return TDSE_OK;
         if (eb != cudaErrorMemoryAllocation) return cuda_error(eb, "tdse_dipole_spectrum");

@@ -74,4 +74,43 @@ inline int j0_table_nodes(double x_max, int64_t n_rho, int64_t n_z, int64_t n_om
     return saved > 1.2 * (75.0 + 0.49 * x) ? (int)std::min(4.0 * x_max + 3.0, (double)kJ0MaxNodes) : 0;
 }
 
+// ---- spectra (tdse_dft.cu)
+
+// Block length and number of moments for n_rows rows of `samples` samples at n_w frequencies that turn by at most
+// `turn` rad a sample; false where the direct sum is the better one: where blocks do not halve its instructions, and
+// for short rows, whose chain of samples is shorter than the moments' kernels.  In us: the direct sum takes 0.235 a
+// sample, or 1.3e-5 a sample and thread once these fill the pipe; the moments 130 + 2.2 P for their tables and weights,
+// a warp's chain over half a block, and a CTA's over the blocks of its 4 rows (k_band), as often as an SM has CTAs.
+// Measured, whole calls, direct and by moments: 64 rows of 512, 60 bins 325 and 547 us; 16 of 1000, 60 446 and 564; 4 of
+// 2000, 120 677 and 737 (60: 676 and 593); 16 of 4000, 400 1154 and 1289 (120: 1151 and 762; 64 rows: 2023 and 1282).
+inline bool dft_plan(int64_t samples, double turn, int64_t n_w, int64_t n_rows, int sm_count, int* B_out, int* P_out)
+{
+    *B_out = *P_out = 0;
+    if (n_w < 32 || samples < 256 || !(turn < 0.8)) return false;
+    double best = 0.5 * 6.0 * (double)n_w;   // the direct sum per sample; the blocks have to halve it
+    int best_B = 0, best_P = 0;
+    for (int B = 32; B <= 1024; B *= 2)
+        for (int P = 16; P <= 40; P += 8) {
+            const double phi = 0.5 * turn * B;
+            if (phi > 0.0 && P * std::log(0.5 * phi) - std::lgamma(P + 1.0) + std::log(2.0) > std::log(1e-17)) continue;
+            const double cost = 0.5 * P + 1.0 + (double)n_w * (P + 6.0) / B;
+            if (cost < best) {
+                best = cost;
+                best_B = B;
+                best_P = P;
+            }
+            break;
+        }
+    if (best_B == 0) return false;
+    const double L = (double)samples, rows = (double)n_rows, B = best_B, P = best_P, sms = std::max(1, sm_count);
+    const double tiles = (double)((n_w + 127) / 128), R = n_rows >= 4 ? 4.0 : 1.0, blocks = std::ceil(L / B);
+    const double direct = L * std::max(0.235, 1.3e-5 * rows * tiles * 128.0);
+    const double moments = 130.0 + 2.2 * P + 0.0083 * B * P * std::max(1.0, rows * blocks / 16.0 / (4.0 * sms)) +
+                           0.0333 * blocks * R * (P + 6.0) * std::max(1.0, tiles * std::ceil(rows / R) / sms);
+    if (moments >= direct) return false;
+    *B_out = best_B;
+    *P_out = best_P;
+    return true;
+}
+
 }  // namespace tdse
