@@ -199,9 +199,9 @@ tdse_status tdse_check(tdse_batch* batch, int64_t* first_bad_host, void* stream)
  *   epsilon       resolution eps >= 1e-12 a.u.
  *   P_dev         out: n_inst x n_energies doubles, row i = instance i in creation order
  * Works on FP64 and MIXED batches (the solves always run in FP64).  Synchronous: allocates the
- * pivot tables (2 x 16 B x N x n_energies per class) for the call, keeps a solve scratch of
- * 16 x SMs x 32 x N_max x 16 B on the batch (8 x where that is above 8 GB), and synchronises the stream
- * before returning. */
+ * pivot tables (16 B x N x n_energies per class, twice that on NUMEROV_SPLIT) for the call, keeps a solve
+ * scratch of 16 x SMs x 32 x N_max x 16 B on the batch (8 x on NUMEROV_SPLIT, where that is above 8 GB or the device
+ * has no room for it; less for few solves), and synchronises the stream before returning. */
 tdse_status tdse_energy_distribution(tdse_batch* batch, const double* E_grid_host, int32_t n_energies,
                                      double epsilon, double* P_dev, void* stream);
 

@@ -1225,13 +1225,21 @@ tdse_status tdse_energy_distribution(tdse_batch* b, const double* E_grid_host, i
         piv_elems += (int64_t)b->classes[c].N * nE_pad;
         n_max = std::max(n_max, b->classes[c].N);
     }
-    const int64_t sc = energy_distribution_scratch_elems(b->sm_count, n_max, (int)b->scheme, b->n_slots, n_energies);
+    int blocks = energy_distribution_blocks(b->sm_count, n_max, (int)b->scheme, b->n_slots, n_energies, true);
+    int64_t sc = energy_distribution_scratch_elems(blocks, n_max, b->n_slots, n_energies);
     if (sc > b->ed_scratch_elems) {
         TDSE_CUDA(cudaStreamSynchronize(st), "tdse_energy_distribution: synchronize");
         cudaFree(b->d_ed_scratch);
         b->d_ed_scratch = nullptr;
         b->ed_scratch_elems = 0;
-        TDSE_CUDA(cudaMalloc(&b->d_ed_scratch, sizeof(double2) * (size_t)sc), "cudaMalloc(energy distribution scratch)");
+        cudaError_t em = cudaMalloc(&b->d_ed_scratch, sizeof(double2) * (size_t)sc);
+        if (em == cudaErrorMemoryAllocation) {   // fewer warps: the same bits, with half of the scratch
+            cudaGetLastError();
+            blocks = energy_distribution_blocks(b->sm_count, n_max, (int)b->scheme, b->n_slots, n_energies, false);
+            sc = energy_distribution_scratch_elems(blocks, n_max, b->n_slots, n_energies);
+            em = cudaMalloc(&b->d_ed_scratch, sizeof(double2) * (size_t)sc);
+        }
+        TDSE_CUDA(em, "cudaMalloc(energy distribution scratch)");
         b->ed_scratch_elems = sc;
     }
     // per-call buffers: energies, pivot tables and their offsets (freed after the stream drains)
@@ -1244,14 +1252,14 @@ tdse_status tdse_energy_distribution(tdse_batch* b, const double* E_grid_host, i
         cudaFree(d_off);
     };
     cudaError_t e = cudaMalloc(&d_E, sizeof(double) * n_energies);
-    if (e == cudaSuccess) e = cudaMalloc(&d_piv, sizeof(double2) * 2 * (size_t)piv_elems);
+    if (e == cudaSuccess) e = cudaMalloc(&d_piv, sizeof(double2) * (b->scheme == TDSE_FULL_CN ? 1 : 2) * (size_t)piv_elems);
     if (e == cudaSuccess) e = cudaMalloc(&d_off, sizeof(int64_t) * n_cls);
     if (e == cudaSuccess) e = cudaMemcpyAsync(d_E, E_grid_host, sizeof(double) * n_energies, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(d_off, piv_off.data(), sizeof(int64_t) * n_cls, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess)
         e = launch_energy_distribution(b->mixed(), b->d_groups, b->d_cls, n_cls, b->d_tab, b->d_slot_group,
                                        b->d_slot_inst, b->n_slots, b->d_psi, d_E, n_energies, epsilon, (int)b->scheme,
-                                       d_piv, d_off, piv_elems, b->d_ed_scratch, n_max, b->sm_count, P_dev, st);
+                                       d_piv, d_off, piv_elems, b->d_ed_scratch, n_max, blocks, P_dev, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     release();
     if (e != cudaSuccess) return cuda_fail(e, "tdse_energy_distribution");

@@ -363,14 +363,16 @@ cudaError_t launch_adjoint_fix(const GroupDesc* d_groups, int64_t n_groups, int 
                                double* gE, int mask_on, int* d_busy, int* d_progress, int* d_left, cudaStream_t st, int have_ckpt);
 
 // Energy distribution of every instance state (tdse_resolvent.cu): pivots per (class, energy) into
-// d_piv (2 * piv_elems complex doubles, class c at d_piv_off[c], N_c rows of nE rounded up to 32),
-// then one warp per (instance, 32 energies) with a scratch of energy_distribution_scratch_elems.
-int64_t energy_distribution_scratch_elems(int sm_count, int n_max, int scheme, int64_t n_slots, int nE);
+// d_piv (piv_elems complex doubles, twice that on NUMEROV_SPLIT; class c at d_piv_off[c], N_c rows of nE rounded up to
+// 32), then one warp per (instance, 32 energies) of `blocks` blocks, with a scratch of
+// energy_distribution_scratch_elems.  energy_distribution_blocks: as many as pay, with `room` for their scratch or not.
+int energy_distribution_blocks(int sm_count, int n_max, int scheme, int64_t n_slots, int nE, bool room);
+int64_t energy_distribution_scratch_elems(int blocks, int n_max, int64_t n_slots, int nE);
 cudaError_t launch_energy_distribution(int mixed, const GroupDesc* d_groups, const ClassDesc* d_cls, int n_cls,
                                        const double* d_tab, const int64_t* d_slot_group, const int64_t* d_slot_inst,
                                        int64_t n_slots, const void* d_psi, const double* d_E_grid, int nE, double eps,
                                        int scheme, void* d_piv, const int64_t* d_piv_off, int64_t piv_elems,
-                                       void* d_scratch, int n_max, int sm_count, double* P_out, cudaStream_t st);
+                                       void* d_scratch, int n_max, int blocks, double* P_out, cudaStream_t st);
 
 // Ionisation probability: out[i] = sum_k w[k] P[i * nE + k] (one warp per instance).
 cudaError_t launch_ionisation(const double* d_P, int64_t n_inst, int nE, const double* d_w, double* d_out,

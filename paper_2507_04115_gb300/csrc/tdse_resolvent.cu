@@ -24,26 +24,19 @@ namespace tdse {
 
 namespace {
 
-// Sub-diagonal, diagonal and super-diagonal of (z M - K) at point j (z = E - i eps), FULL_CN or
-// NUMEROV_SPLIT; V from the class table.
+// Sub-diagonal, diagonal and super-diagonal of (z M2 - K) at point j (z = E - i eps), NUMEROV_SPLIT; V from the class
+// table.
 struct EdRow {
     double2 a, b, c;
 };
 
-__device__ __forceinline__ EdRow ed_row(int scheme, double zr, double zi, double inv_dx2, const double* __restrict__ V,
-                                        int j, int N)
+__device__ __forceinline__ EdRow ed_row(double zr, double zi, double inv_dx2, const double* __restrict__ V, int j, int N)
 {
     EdRow r;
-    if (scheme == 0) {
-        r.a = make_double2(j > 0 ? 0.5 * inv_dx2 : 0.0, 0.0);
-        r.c = make_double2(j < N - 1 ? 0.5 * inv_dx2 : 0.0, 0.0);
-        r.b = make_double2(zr - (inv_dx2 + V[j]), zi);
-    } else {
-        const double k12 = 1.0 / 12.0;
-        r.a = j > 0 ? make_double2(fma(zr, k12, 0.5 * inv_dx2 - V[j - 1] * k12), zi * k12) : make_double2(0.0, 0.0);
-        r.c = j < N - 1 ? make_double2(fma(zr, k12, 0.5 * inv_dx2 - V[j + 1] * k12), zi * k12) : make_double2(0.0, 0.0);
-        r.b = make_double2(fma(zr, 10.0 * k12, -(inv_dx2 + 10.0 * k12 * V[j])), zi * (10.0 * k12));
-    }
+    const double k12 = 1.0 / 12.0;
+    r.a = j > 0 ? make_double2(fma(zr, k12, 0.5 * inv_dx2 - V[j - 1] * k12), zi * k12) : make_double2(0.0, 0.0);
+    r.c = j < N - 1 ? make_double2(fma(zr, k12, 0.5 * inv_dx2 - V[j + 1] * k12), zi * k12) : make_double2(0.0, 0.0);
+    r.b = make_double2(fma(zr, 10.0 * k12, -(inv_dx2 + 10.0 * k12 * V[j])), zi * (10.0 * k12));
     return r;
 }
 
@@ -91,7 +84,7 @@ __global__ void k_ed_pivots(const ClassDesc* __restrict__ cls, int n_cls, const 
     }
     double2 cprev = make_double2(0.0, 0.0);
     for (int j = 0; j < N; ++j) {
-        const EdRow r = ed_row(scheme, zr, zi, inv_dx2, V, j, N);
+        const EdRow r = ed_row(zr, zi, inv_dx2, V, j, N);
         const double2 ac = cmul(r.a, cprev);
         const double2 w = make_double2(r.b.x - ac.x, r.b.y - ac.y);
         const double2 iw = cinv(w);
@@ -240,36 +233,36 @@ cudaError_t launch_ionisation(const double* d_P, int64_t n_inst, int nE, const d
 }
 
 // Blocks of 8 warps, one warp per task (slot, 32 energies) at a time.  FULL_CN: 2 an SM, as a warp's two dependent sweeps
-// leave the FP64 pipe idle for half of the time with one, while their scratch stays below 8 GB; the Numerov pencil, whose
-// rows have more independent work, gained 0.5 % from it (8.15 and 8.11 ms): 1.  Fewer tasks than warps: spread over the
-// blocks, and no more scratch (which the first call allocates) than tasks.
-static int solve_blocks(int sm_count, int n_max, int scheme, int64_t tasks)
+// leave the FP64 pipe idle for half of the time with one, while their scratch stays below 8 GB and the device has room
+// for it (`room`); the Numerov pencil, whose rows have more independent work, gained 0.5 % from it (8.15 and 8.11 ms): 1.
+// Fewer tasks than warps: spread over the blocks, and no more scratch (which the first call allocates) than tasks.
+int energy_distribution_blocks(int sm_count, int n_max, int scheme, int64_t n_slots, int nE, bool room)
 {
-    const bool two = scheme == 0 && (int64_t)sm_count * 16 * kLanes * n_max * (int64_t)sizeof(double2) <= (int64_t(8) << 30);
+    const int64_t tasks = n_slots * ((nE + kLanes - 1) / kLanes);
+    const bool two = room && scheme == 0 && (int64_t)sm_count * 16 * kLanes * n_max * (int64_t)sizeof(double2) <= (int64_t(8) << 30);
     return (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)sm_count * (two ? 2 : 1), tasks));
 }
 
-int64_t energy_distribution_scratch_elems(int sm_count, int n_max, int scheme, int64_t n_slots, int nE)
+int64_t energy_distribution_scratch_elems(int blocks, int n_max, int64_t n_slots, int nE)
 {
     const int64_t tasks = n_slots * ((nE + kLanes - 1) / kLanes);
-    return std::max<int64_t>(1, std::min<int64_t>((int64_t)solve_blocks(sm_count, n_max, scheme, tasks) * 8, tasks)) * kLanes * n_max;
+    return std::max<int64_t>(1, std::min<int64_t>((int64_t)blocks * 8, tasks)) * kLanes * n_max;
 }
 
 cudaError_t launch_energy_distribution(int mixed, const GroupDesc* d_groups, const ClassDesc* d_cls, int n_cls,
                                        const double* d_tab, const int64_t* d_slot_group, const int64_t* d_slot_inst,
                                        int64_t n_slots, const void* d_psi, const double* d_E_grid, int nE, double eps,
                                        int scheme, void* d_piv, const int64_t* d_piv_off, int64_t piv_elems,
-                                       void* d_scratch, int n_max, int sm_count, double* P_out, cudaStream_t st)
+                                       void* d_scratch, int n_max, int blocks, double* P_out, cudaStream_t st)
 {
     if (nE == 0 || n_slots == 0) return cudaSuccess;
     const int nE_pad = (nE + kLanes - 1) / kLanes * kLanes;
-    double2* pivW = static_cast<double2*>(d_piv);
-    double2* pivC = pivW + piv_elems;
+    double2* pivC = static_cast<double2*>(d_piv);
+    double2* pivW = scheme == 0 ? nullptr : pivC + piv_elems;   // (FULL_CN: one table)
     dim3 pg((nE_pad + 127) / 128, n_cls);
     k_ed_pivots<<<pg, 128, 0, st>>>(d_cls, n_cls, d_tab, d_E_grid, nE, nE_pad, eps, scheme, pivW, pivC, d_piv_off);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const int blocks = solve_blocks(sm_count, n_max, scheme, n_slots * (nE_pad / kLanes));
     auto solve = [&](auto kernel, auto psi) {
         kernel<<<blocks, 256, 0, st>>>(d_groups, d_cls, d_tab, d_slot_group, d_slot_inst, n_slots, psi, d_E_grid, nE, nE_pad, eps,
                                        pivW, pivC, d_piv_off, static_cast<double2*>(d_scratch), n_max, P_out);
