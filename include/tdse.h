@@ -381,9 +381,9 @@ tdse_status tdse_set_wait_limit(tdse_batch* batch, int64_t polls);
  * each instance's tridiagonal solve is split into, i.e. the depth of the parallel split), CTAs per
  * SM and the scheduling slice.  It times tdse_propagate over steps [step_begin, step_end) of the
  * given field rows (same arguments as tdse_propagate) for each candidate, every trial starting
- * from the batch's current state, which is restored afterwards: a coordinate search over
- * warps {4, 6, 8, 12, 16} x CTAs per SM {1, 2} at a 16-step slice, then slices {8, 32, 64} at the
- * best pair; shapes that the occupancy clamp makes identical are timed once.  The fastest shape
+ * from the batch's current state, which is restored afterwards: a coordinate search over the default
+ * launch, warps {4, 6, 8, 12, 16} x CTAs per SM {1, 2} and 4 x 4 at a 16-step slice (1 CTA per SM alone
+ * where the longest group bounds the job), then slices {8, 32, 64} at the best of these; shapes that the occupancy clamp makes identical are timed once.  The fastest shape
  * stays set on the batch.
  *   d_dev, a_dev    rows over the probed steps are scratch: overwritten by the probes
  *   repeats         timed runs per candidate in [1, 100] (the minimum counts); the first

@@ -130,6 +130,7 @@ struct tdse_batch {
     size_t gtape_bytes = 0;
     bool use_gtape = true;             // tdse_set_adjoint_gamma_tape
     int adj_kc = 0, adj_ctas = 0;
+    int per_sm = 1;                    // CTAs per SM of the launch
     bool any_fix = false;              // a class of the batch has the fixed-point form
     // launch shapes of the adjoint kernels (one CTA per SM): the fixed-point one by that sweep's rules, the FP64 one with
     // the groups' split for the FP64 sweeps
@@ -570,6 +571,7 @@ tdse_status build_plan(tdse_batch* b)
         const int64_t n = std::min<int64_t>((int64_t)b->groups.size(), (int64_t)b->sm_count * k);
         return (int)(b->max_ctas_override > 0 ? std::min<int64_t>(n, b->max_ctas_override) : n);
     };
+    b->per_sm = per_sm;
     b->ctas = grid(per_sm);
     int64_t sc = (int64_t)b->ctas * b->warps * b->rows * 2 * kLanes;
     if (b->precision == TDSE_FP64 && b->scheme == TDSE_FULL_CN) {
@@ -717,6 +719,7 @@ tdse_status adjoint_launches(tdse_batch* b, const double* E, const double* gd, c
 
 namespace tdse {
 int batch_device(const tdse_batch* b) { return b->device; }
+int batch_ctas_per_sm(const tdse_batch* b) { return b->per_sm; }
 }  // namespace tdse
 
 extern "C" {

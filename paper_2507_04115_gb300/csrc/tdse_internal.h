@@ -296,6 +296,7 @@ const char* set_error_message(const char* msg);
 
 // CUDA device a batch was created on (for host code layered on the public calls).
 int batch_device(const tdse_batch* b);
+int batch_ctas_per_sm(const tdse_batch* b);
 
 // ---- kernel launchers (tdse_kernels.cu); all return cudaGetLastError() after the launch ----
 

@@ -7,7 +7,8 @@ kind of batch without timing again.  This module keeps such shapes in a JSON fil
 
     {"version": 1, "shapes": {<key>: {"warps_per_cta": W, "ctas_per_sm": C, "slice_steps": S}}}
 
-Keys are canonical JSON strings of the quantities above.  Writes go to a temporary file in the
+Keys are canonical JSON strings of the quantities above and of the generation of the propagation kernels, so that a
+shape found for other kernels is not applied to these.  Writes go to a temporary file in the
 same directory that then replaces the table, so a reader never sees a partial file.  Host logic
 only: applying a shape is one tdse_set_launch call, exactly what the autotuner does with its
 fastest trial.
@@ -18,6 +19,7 @@ import json
 import os
 import tempfile
 
+SWEEPS = 2   # the propagation kernels whose shapes are stored (2: the fixed-point sweeps)
 SHAPE_FIELDS = ("warps_per_cta", "ctas_per_sm", "slice_steps")
 
 
@@ -26,7 +28,7 @@ def batch_key(classes, precision, scheme, lanes_per_instance, gpu_name) -> str:
     of the classes does not matter."""
     cls = sorted((int(N), float(dx), float(a), float(Z), int(c)) for N, dx, a, Z, c in classes)
     payload = {"classes": cls, "precision": int(precision), "scheme": int(scheme),
-               "lanes": int(lanes_per_instance), "gpu": str(gpu_name)}
+               "lanes": int(lanes_per_instance), "gpu": str(gpu_name), "sweeps": SWEEPS}
     return json.dumps(payload, sort_keys=True, separators=(",", ":"))
 
 
