@@ -21,7 +21,8 @@
 //   gamma  2^64 in products (|gamma| <= beta <= 0.35), 2^58 in the pivot recurrence
 //   Q, S   2^58, |Re Q|, |Im Q| < 16 for every |E| <= E_lim
 // With a 2-norm near 2^60.5 one unit is 2^-60.5 of it; spread over N points, its rounding stays below
-// that of the same sweep in double (tests/test_fixed_point_sweep.py measures both against 113 bits).
+// that of the same sweep in double (tests/test_fixed_point_sweep.py and test_fixed_point_forms.py measure both against
+// 113 bits).
 #pragma once
 
 #include <algorithm>
@@ -153,6 +154,43 @@ __host__ __device__ __forceinline__ int64_t update_fix(int32_t ci, Digits cf, Di
     return fold(mad(cf.h, y.h, acc), mad(cf.h, y.l, mad(cf.l, y.h, int64_t(1) << 31)));
 }
 
+// ---- NUMEROV_SPLIT (tdse_numerov_fix.cuh)
+
+// (a b + c d) 2^-62, rounded
+__host__ __device__ __forceinline__ int64_t mul2_fix62(Digits a, Digits b, Digits c, Digits d)
+{
+    return combine<2, 30>(mad(a.h, b.h, mad(c.h, d.h, 0)),
+                          mad(a.h, b.l, mad(a.l, b.h, mad(c.h, d.l, mad(c.l, d.h, int64_t(1) << 29)))));
+}
+
+// cos and sin of `turn` 2^-64 turns at 2^62, within a few units: the angle reduced to [-1/8, 1/8] turn and
+// the Taylor polynomials to theta^18 and theta^19 (next term 3e-21), in fixed point: about 250
+// instructions, where sincos takes about 50 FP64 instructions of 64 cycles.
+__host__ __device__ __forceinline__ void fix_cos_sin(uint64_t turn, int64_t& c, int64_t& s)
+{
+    const int quad = (int)((turn + (uint64_t(1) << 61)) >> 62);
+    const int64_t r = (int64_t)(turn - ((uint64_t)quad << 62));            // |r| <= 2^61
+    const Digits th = digits(mul_fix<3>(digits(r), digits(3622009729038561421)));   // pi/2 2^61: theta at 2^62
+    const Digits z = digits(mul_fix<2>(th, th));
+    // (-1)^k / (2k)! and (-1)^k / (2k+1)! at 2^62
+    const int64_t kc[10] = {4611686018427387904, -2305843009213693952, 192153584101141163, -6405119470038039, 114377133393536,
+                            -1270857037706, 9627704831, -52899477, 220414, -720};
+    const int64_t ks[10] = {4611686018427387904, -768614336404564651, 38430716820228233, -915017067148291, 12708570377060,
+                            -115532457973, 740592679, -3526632, 12966, -38};
+    int64_t a = kc[9], b = ks[9];
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+    for (int k = 8; k >= 0; --k) {
+        a = kc[k] + mul_fix<2>(z, digits(a));
+        b = ks[k] + mul_fix<2>(z, digits(b));
+    }
+    b = mul_fix<2>(th, digits(b));
+    const int64_t c0 = (quad & 1) ? -b : a, s0 = (quad & 1) ? a : b;
+    c = (quad & 2) ? -c0 : c0;
+    s = (quad & 2) ? -s0 : s0;
+}
+
 __host__ __device__ __forceinline__ float rcp_f32(float x)
 {
 #ifdef __CUDA_ARCH__
@@ -167,7 +205,8 @@ __host__ __device__ __forceinline__ float rcp_f32(float x)
 // 2^116 / n for n in [2^55, 2^61): float seed r0 ~ 2^85 / n (|relative error e| < 2^-22) and one
 // third-order Newton step.  e is carried in units of 2^-53 and below that, with e^2, in units of 2^-61
 // (to 2^-53 alone its rounding acts alike on every step near the nucleus, and the error of the sweep
-// grows with the number of steps): the result is within 2^-55 relative.
+// grows with the number of steps): the result is within 2^-55 relative for n < 2^59 (|Q|^2 < 128), 2^-53 up to the
+// end of the range, where the floors of the three terms, all one way, add up (tests/test_fixed_point_forms.py).
 __host__ __device__ __forceinline__ int64_t recip_fix(int64_t n)
 {
     const uint32_t nl = (uint32_t)(uint64_t)n, nh = (uint32_t)((uint64_t)n >> 32);
