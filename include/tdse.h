@@ -60,8 +60,12 @@ typedef enum {
 typedef enum {
     TDSE_FP64 = 0,   /* the wavefunctions in IEEE double between calls; within a call the steps and the
                         observable sums in 64-bit fixed point (60 bits of an instance's norm, gamma to
-                        2^-58; error not above that of the sweep in double), for dt/(4 dx^2) in [0.0715, 0.35]
-                        (FULL_CN), N <= 32768, usual fields and norms; otherwise, per slice of a group, the
+                        2^-53 of itself; error not above that of the sweep in double).  Its range:
+                        N <= 32768, instance norms sqrt(sum |psi_j|^2) from 1e-15 to 1e15, and FULL_CN
+                        dt / (4 dx^2) in [0.0715, 0.35] and fields to about 13 / (N dx^3) (0.94 a.u. at
+                        N = 4096, dx = 0.15; 0.20, 0.10 and 0.05 at dx = 0.2 and N = 8192, 16384 and 32768),
+                        NUMEROV_SPLIT dt / dx^2 to about 1.5 (factors decaying by 0.35 a point).  A class
+                        outside it, or a slice of a group of which one field or norm is, takes the
                         solve in double and |psi|^2 and the sums as float pairs (about 2^-44 relative per
                         point) over blocks of 16 points, added in double across blocks */
     TDSE_MIXED = 1   /* psi, the solve's right-hand side and back substitution in float; the
