@@ -529,7 +529,7 @@ int shape_groups(const tdse_batch* b, std::vector<GroupDesc>& groups, bool fix, 
     if (b->warps_override > 0) *widest = most;
     for (auto& G : groups) {
         const int L = kLanes / G.I;
-        G.P64 = G.P;
+        G.P64 = (int16_t)G.P;
         G.m64 = G.m;
         if (fix && on_fix_path(b, b->classes[G.cls])) fp64_split(G.N, G.K, G.P, L, std::min(most, *widest), &G.P64, &G.m64);
         // the FP64 sweeps pack their P64 warps' rows into the CTA's scratch, *widest x rows

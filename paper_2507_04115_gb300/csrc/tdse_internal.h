@@ -54,12 +54,13 @@ struct GroupDesc {
     int64_t nt_max;       // largest Nt over the group's real instances
     int32_t cls;          // class index
     int32_t N, P, K, m;   // grid size, warps carrying segments, halo, segment length
-    int32_t I;            // instances per group (32, 16, 8, 4, 2 or 1)
+    int16_t I;            // instances per group (32, 16, 8, 4, 2 or 1)
+    int16_t P64;          // warps and segment length of the FP64 sweeps (P and m where the group has no
+    int32_t m64;          // fixed-point form): slices outside the fixed-point range run at these
     int32_t w;            // cost of one time step (units of group_step_cost / 64, >= 1): the
                           // scheduler's priority is remaining slices x w
-    int32_t P64, m64;     // warps and segment length of the FP64 sweeps (P and m where the group has
-                          // no fixed-point form): slices outside the fixed-point range run at these
 };
+static_assert(sizeof(GroupDesc) == 56, "the static entry point's scratch holds one per 32 instances");
 
 // Device-side tables offsets inside a class block (in doubles).  Tables are laid out at the grid size
 // rounded up to even, so that every table (an odd multiple of it among them) starts on the 16 bytes
@@ -171,11 +172,11 @@ inline int fix_warps(int N, int K, int L, int warps, int per_sm, double lead)
 // hide.  Measured, fields beyond the range, warps of the fixed-point split and 8: 300 instances of 2048 points at
 // 16 lanes, 64 steps, 9.75 ms at 10 and 8.27 (cost 0.70); 64 of 8192 at 32 lanes 13.0 at 16 and 9.5 (0.65);
 // 2048 of 16384 at 4 lanes 35.9 at 16 and 45.4 (0.95); 8192 of 4096 at 1 lane 64.6 at 16 and 64.3 (0.94).
-inline void fp64_split(int N, int K, int P, int L, int warps, int32_t* P64, int32_t* m64)
+inline void fp64_split(int N, int K, int P, int L, int warps, int16_t* P64, int32_t* m64)
 {
     auto cost = [&](int p) { return std::ceil(p / 4.0) * (27.0 * group_segment_length(N, p, L) + 36.0 * (p * L > 1 ? K : 0)); };
     const int rule = P == 1 && L == 1 ? 1 : group_warps(N, K, L, warps);   // (P == 1, L == 1: one exact segment, planned without a halo)
-    *P64 = cost(rule) < 0.8 * cost(P) ? rule : P;
+    *P64 = (int16_t)(cost(rule) < 0.8 * cost(P) ? rule : P);
     *m64 = group_segment_length(N, *P64, L);
 }
 

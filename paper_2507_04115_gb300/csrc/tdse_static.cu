@@ -65,7 +65,7 @@ __global__ void k_static_setup(ClassDesc C, int64_t n_inst, int64_t n_groups, in
         G.P = P;
         G.K = K;
         G.m = m;
-        G.P64 = P;
+        G.P64 = (int16_t)P;
         G.m64 = m;
         G.I = kLanes;
         G.w = 1;
@@ -158,9 +158,12 @@ extern "C" tdse_status tdse_propagate_static(const tdse_instance* inst_host, int
     const size_t o_busy = take(sizeof(int) * (size_t)n_groups);
     const size_t o_prog = take(sizeof(int) * (size_t)n_groups);
     const size_t o_status = take(sizeof(int) * (size_t)n_groups * kLanes);
-    const size_t o_tab = take(sizeof(double) * (size_t)tab_doubles(C));
-    const size_t o_scratch = off;
+    const size_t o_tab = off;
     const size_t per_cta = sizeof(double2) * (size_t)warps * rows * 2 * kLanes;
+    // (the fixed-point form's tables take more room: without it where that is what is missing)
+    if (C.fix.ok && align256(o_tab + sizeof(double) * (size_t)tab_doubles(C)) + per_cta > kStaticBytes) C.fix.ok = 0;
+    take(sizeof(double) * (size_t)tab_doubles(C));
+    const size_t o_scratch = off;
     if (o_scratch >= kStaticBytes || (kStaticBytes - o_scratch) / per_cta < 1) {
         static thread_local char msg[256];
         std::snprintf(msg, sizeof msg,
