@@ -517,7 +517,7 @@ int shape_groups(const tdse_batch* b, std::vector<GroupDesc>& groups, bool fix, 
         const int cap = fix && b->warps_override <= 0 ? std::min(most, most_fix) : most;
         const int P = fx ? fix_warps(C.N, K, L, most_fix, per_sm, fix_lead(b)) : group_warps(C.N, K, L, cap);
         if (P == 1 && L == 1) K = 0;   // one exact segment
-        G.P = P;
+        G.P = (int16_t)P;
         G.K = K;
         G.m = group_segment_length(G.N, P, L);
         G.w = std::max(1, (int)std::lround((fx ? fix_step_cost(C.N, K, L, P, P * per_sm, fix_lead(b)) : group_step_cost(C.N, K, L, cap)) / 64.0));
@@ -561,7 +561,7 @@ tdse_status build_plan(tdse_batch* b)
     b->class_P.assign(n_cls, 1);
     b->class_K.assign(n_cls, 0);
     for (const GroupDesc& G : b->groups) {
-        b->class_P[G.cls] = std::max(b->class_P[G.cls], G.P);
+        b->class_P[G.cls] = std::max<int>(b->class_P[G.cls], G.P);
         b->class_K[G.cls] = std::max(b->class_K[G.cls], G.K);
     }
     const int per_sm_max = propagate_max_ctas_per_sm(b->mixed(), fix, b->warps);
@@ -584,7 +584,7 @@ tdse_status build_plan(tdse_batch* b)
         for (GroupDesc& G : b->adj_groups) {
             G.P = G.P64;
             G.m = G.m64;
-            b->adj_warps = std::max(b->adj_warps, G.P);
+            b->adj_warps = std::max<int>(b->adj_warps, G.P);
             b->adj_rows = std::max(b->adj_rows, G.P * (kLanes / G.I) == 1 ? G.N : G.m + 2 * G.K);
         }
         b->adj_grid = grid(b->ctas_per_sm_override > 0 ? std::min(b->ctas_per_sm_override, propagate_max_ctas_per_sm(0, fix, std::max(b->adj_warps, b->adj_fix_warps))) : 1);

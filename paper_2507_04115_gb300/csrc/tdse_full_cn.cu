@@ -710,7 +710,7 @@ cudaError_t launch_propagate_full_cn(int mixed, int fix, const GroupDesc* d_grou
     e = cudaMemsetAsync(d_progress, 0, sizeof(int) * n_groups, st);
     if (e != cudaSuccess) return e;
     if (mixed && (ring < kMinRing || ring > kMaxRing)) return cudaErrorInvalidValue;
-    const size_t smem = full_cn_smem_bytes(mixed, fix, P, ring);
+    const size_t smem = full_cn_smem_bytes(mixed, P, ring, fix);
     if (mixed) {
         static std::atomic<bool> attr_set[kMaxAttrDevices];
         int dev = 0;
@@ -740,7 +740,7 @@ int propagate_ring_slots(int P, int per_sm) { return full_cn_ring_slots(P, per_s
 int propagate_max_ctas_per_sm(int mixed, int fix, int P)
 {
     int n = 0;
-    const size_t smem = full_cn_smem_bytes(mixed, fix, P, kMinRing);   // the shallowest ring
+    const size_t smem = full_cn_smem_bytes(mixed, P, kMinRing, fix);   // the shallowest ring
     if (mixed &&
         cudaFuncSetAttribute(k_propagate_full_cn<true, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)full_cn_smem_max_bytes()) != cudaSuccess) {

@@ -53,10 +53,11 @@ struct GroupDesc {
     int64_t slot0;        // first slot (slot = slot0 + instance index within the group)
     int64_t nt_max;       // largest Nt over the group's real instances
     int32_t cls;          // class index
-    int32_t N, P, K, m;   // grid size, warps carrying segments, halo, segment length
-    int16_t I;            // instances per group (32, 16, 8, 4, 2 or 1)
-    int16_t P64;          // warps and segment length of the FP64 sweeps (P and m where the group has no
-    int32_t m64;          // fixed-point form): slices outside the fixed-point range run at these
+    int32_t N;            // grid size
+    int16_t P, P64;       // warps carrying segments; those of the FP64 sweeps (with m64 the split of slices
+                          // outside the fixed-point range; P and m where the group has no such form)
+    int32_t K, m, m64;    // halo, segment length, that of the FP64 sweeps
+    int32_t I;            // instances per group (32, 16, 8, 4, 2 or 1)
     int32_t w;            // cost of one time step (units of group_step_cost / 64, >= 1): the
                           // scheduler's priority is remaining slices x w
 };

@@ -35,7 +35,7 @@ inline int full_cn_ring_slots(int P, int per_sm)
 // Values that leave a segment of the fixed-point sweep's short-segment form, per lane (FixEdge).
 constexpr int kEdgeBytes = 48;
 
-__host__ __device__ inline size_t full_cn_smem_bytes(int mixed, int fix, int P, int ring)
+__host__ __device__ inline size_t full_cn_smem_bytes(int mixed, int P, int ring, int fix = 1)
 {
     size_t b = (size_t)P * 3 * 32 * sizeof(double);
     if (!mixed && fix) b += (size_t)P * 32 * kEdgeBytes;
@@ -48,7 +48,7 @@ inline size_t full_cn_smem_max_bytes()
 {
     size_t m = 0;
     for (int P = 1; P <= 16; ++P) {
-        const size_t b = full_cn_smem_bytes(1, 0, P, full_cn_ring_slots(P, 1));
+        const size_t b = full_cn_smem_bytes(1, P, full_cn_ring_slots(P, 1));
         m = b > m ? b : m;
     }
     return m;

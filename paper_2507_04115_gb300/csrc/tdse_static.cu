@@ -62,7 +62,7 @@ __global__ void k_static_setup(ClassDesc C, int64_t n_inst, int64_t n_groups, in
         G.nt_max = nt;
         G.cls = 0;
         G.N = C.N;
-        G.P = P;
+        G.P = (int16_t)P;
         G.K = K;
         G.m = m;
         G.P64 = (int16_t)P;
