@@ -180,9 +180,7 @@ void free_device(tdse_batch* b)
     cudaFree(b->d_slot_inst);
     cudaFree(b->d_ed_scratch);
     cudaFree(b->d_adj_groups);
-    b->d_adj_groups = nullptr;
-    cudaFree(b->d_adj_fix_groups);
-    b->d_adj_fix_groups = nullptr;
+    b->d_adj_groups = b->d_adj_fix_groups = nullptr;
     cudaFree(b->d_left);
     b->d_left = nullptr;
     b->d_slot_group = b->d_slot_inst = nullptr;
@@ -594,20 +592,11 @@ tdse_status build_plan(tdse_batch* b)
             if (on_fix_path(b, b->classes[G.cls]) && G.K > 0)
                 b->adj_fix_scratch = std::max(b->adj_fix_scratch, adjoint_fix_scratch(b->adj_fix_warps, G.m));
         sc = std::max(sc, (int64_t)b->adj_grid * b->adj_fix_scratch);
-        cudaFree(b->d_left);
-        b->d_left = nullptr;
-        TDSE_CUDA(dev_alloc(&b->d_left, b->adj_groups.size()), "cudaMalloc(sched)");
+        // (on the device with the first adjoint call: most batches never make one)
         cudaFree(b->d_adj_groups);
-        b->d_adj_groups = nullptr;
-        TDSE_CUDA(dev_alloc(&b->d_adj_groups, b->adj_groups.size()), "cudaMalloc(groups)");
-        TDSE_CUDA(cudaMemcpy(b->d_adj_groups, b->adj_groups.data(), sizeof(GroupDesc) * b->adj_groups.size(), cudaMemcpyHostToDevice),
-                  "cudaMemcpy(groups)");
-        cudaFree(b->d_adj_fix_groups);
-        b->d_adj_fix_groups = nullptr;
-        TDSE_CUDA(dev_alloc(&b->d_adj_fix_groups, b->adj_fix_groups.size()), "cudaMalloc(groups)");
-        TDSE_CUDA(cudaMemcpy(b->d_adj_fix_groups, b->adj_fix_groups.data(), sizeof(GroupDesc) * b->adj_fix_groups.size(),
-                             cudaMemcpyHostToDevice),
-                  "cudaMemcpy(groups)");
+        cudaFree(b->d_left);
+        b->d_adj_groups = b->d_adj_fix_groups = nullptr;
+        b->d_left = nullptr;
     }
     cudaFree(b->d_scratch);
     b->d_scratch = nullptr;
@@ -697,6 +686,14 @@ tdse_status adjoint_launches(tdse_batch* b, const double* E, const double* gd, c
                              cudaStream_t st, int have_ckpt)
 {
     const int64_t n = (int64_t)b->groups.size();
+    if (!b->d_adj_groups) {   // one array: the FP64 kernel's groups, then the fixed-point one's
+        const size_t bytes = sizeof(GroupDesc) * (size_t)n;
+        TDSE_CUDA(dev_alloc(&b->d_left, (size_t)n), "cudaMalloc(sched)");
+        TDSE_CUDA(dev_alloc(&b->d_adj_groups, 2 * (size_t)n), "cudaMalloc(groups)");
+        b->d_adj_fix_groups = b->d_adj_groups + n;
+        TDSE_CUDA(cudaMemcpy(b->d_adj_groups, b->adj_groups.data(), bytes, cudaMemcpyHostToDevice), "cudaMemcpy(groups)");
+        TDSE_CUDA(cudaMemcpy(b->d_adj_fix_groups, b->adj_fix_groups.data(), bytes, cudaMemcpyHostToDevice), "cudaMemcpy(groups)");
+    }
     int* left = nullptr;
     if (b->adj_fix_scratch > 0 && kc < n_max) {
         left = b->d_left;
