@@ -13,8 +13,8 @@
 // The solve with A_n reuses the forward kernel's segmented, halo-truncated Thomas sweep.
 //
 // Groups within the fixed-point range are served by tdse_adjoint_fix.cu (44.4 -> 14.7 ms at 1024 x 2048 points, 96
-// steps); this kernel runs behind it for the others, or alone when no class has that form or the checkpoint
-// interval is as long as the largest grid.
+// steps); this kernel runs behind it for the others (68.8 ms for all of that batch, from the start), or alone when no
+// class has that form or the checkpoint interval is as long as the largest grid.
 //
 // Memory: the forward states are recomputed from checkpoints every K steps; within a checkpoint
 // interval the pre-mask states psi~ are kept on a per-CTA tape.  One CTA owns a group for the whole

@@ -20,8 +20,8 @@
 //   J0 comes from a table of its Taylor coefficients at the nodes x_i = i / 4 (k_j0_table, filled per call up
 // to the largest argument, where j0_table_nodes finds that it pays): |x - x_i| <= 1/8 and |J0^(n)| <= 1, so 12 terms
 // leave (1/8)^12 / 12! < 4e-20.  A term then costs 17 FP64 instructions (argument, node, 11 of the polynomial, 2 sums);
-// CUDA's j0 takes about 120 beyond x = 8.  Measured, 32 x 32 points, 340 frequencies, 256 radii: 7.1 ms with j0 and
-// 3.4 with the table at arguments up to 20, 14.9 and 3.7 up to 500.
+// CUDA's j0 takes about 120 beyond x = 8.  Measured, 32 x 32 points, 340 frequencies, 256 radii, whole calls: 7.2 ms
+// with j0 and 3.6 with the table at arguments up to 20, 14.4 and 3.9 up to 500.
 #include "tdse.h"
 #include "tdse_internal.h"
 

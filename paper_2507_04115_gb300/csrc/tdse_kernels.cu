@@ -134,7 +134,7 @@ __device__ void block_recurrence(double* __restrict__ x, const double* __restric
 // iteration, one more for the energy, which is formed only where the stopping rule can use it
 // (tol > 0, or the last iteration).
 // Measured, 8 classes of 1024 to 8192 points, 600 iterations: 116 ms with one CTA of 1024 threads per class
-// (a scan of 10 levels per sweep, V and the division by the norm evaluated per point), 2.6 ms here.
+// (a scan of 10 levels per sweep, V and the division by the norm evaluated per point), 6.2 ms here.
 constexpr int kGsCluster = 8;
 constexpr int kGsCtaThreads = 128;
 constexpr int kGsPer = 8;
