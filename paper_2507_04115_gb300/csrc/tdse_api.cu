@@ -680,15 +680,15 @@ void ensure_gamma_tape(tdse_batch* b, int kc)
 
 // The adjoint's kernels: the fixed-point one where a class has that form, then the FP64 one for what it leaves (all
 // groups when no class has it, or the interval is too long for its per-sample sums) at its own shape and with its gamma
-// tape: with fields beyond the range, 1024 x 2048 points, 96 steps, an interval of 32, it takes 68.8 ms
-// so, and 92.6 at the fixed-point shape without the tape.
+// tape: with fields beyond the range, 1024 x 2048 points, 96 steps, an interval of 32, it takes 68.8 ms so, and 92.6 at
+// the fixed-point shape without the tape.
 tdse_status adjoint_launches(tdse_batch* b, const double* E, const double* gd, const double* ga, double* gE, int n_max, int kc,
                              cudaStream_t st, int have_ckpt)
 {
     const int64_t n = (int64_t)b->groups.size();
     if (!b->d_adj_groups) {   // one array: the FP64 kernel's groups, then the fixed-point one's
         const size_t bytes = sizeof(GroupDesc) * (size_t)n;
-        TDSE_CUDA(dev_alloc(&b->d_left, (size_t)n), "cudaMalloc(sched)");
+        if (!b->d_left) TDSE_CUDA(dev_alloc(&b->d_left, (size_t)n), "cudaMalloc(sched)");
         TDSE_CUDA(dev_alloc(&b->d_adj_groups, 2 * (size_t)n), "cudaMalloc(groups)");
         b->d_adj_fix_groups = b->d_adj_groups + n;
         TDSE_CUDA(cudaMemcpy(b->d_adj_groups, b->adj_groups.data(), bytes, cudaMemcpyHostToDevice), "cudaMemcpy(groups)");

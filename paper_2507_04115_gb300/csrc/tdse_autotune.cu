@@ -11,7 +11,8 @@
 //                   work queue (load balance vs. scheduling overhead).
 // The search is coordinate-wise: the default launch and (warps, CTAs per SM) over a small grid first, then the slice at
 // the best of these.  The default is the planner's for the batch (it takes 625 groups of 1024 points at 4 CTAs of 4
-// warps, 26.4 ms, where 2 of 8 take 29.1), so that a tuned batch is not slower than an untuned one.  Every trial starts from the same saved state; the state is put back at the end.
+// warps, 26.4 ms, where 2 of 8 take 29.1), so that a tuned batch is not slower than an untuned one.  Every trial starts
+// from the same saved state; the state is put back at the end.
 #include "tdse.h"
 #include "tdse_internal.h"
 
